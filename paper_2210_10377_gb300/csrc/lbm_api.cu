@@ -14,6 +14,7 @@
 
 #include "lbm_host.h"
 #include "lbm_internal.cuh"
+#include "lbm_march.cuh"
 
 using namespace gblbm;
 
@@ -42,6 +43,12 @@ constexpr double ADJ_KEEP_SHARE = GBLBM_ADJ_KEEP_SHARE;
 #define GBLBM_BODY_ROWS_FIRST 1
 #endif
 constexpr int TIMING_BATCH = 64;
+// Multi-step passes per captured graph: long and short form (multiples of
+// NBUF, so that a graph ends on the buffer it starts from).
+constexpr int GRAPH_PASSES[2] = {12, NBUF};
+// Share of the grid that the kept intermediate states may cover: with more of
+// it the pass writes so much that single steps are as fast.
+constexpr double MARCH_KEEP_SHARE = 0.25;
 
 }  // namespace
 
@@ -72,10 +79,23 @@ struct lbm_ctx {
     cudaStream_t side = nullptr; // link kernels
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_read[NBUF] = {nullptr, nullptr, nullptr};
     bool ev_live[NBUF] = {false, false, false};
-    // The step whose collide-stream kernel is queued and whose link kernel is
-    // not yet (lead_src < 0: none): it goes out beside the next step's
-    // collide-stream kernel, or when the queue ends.
-    int lead_src = -1, lead_pre = 0;
+    // The step or pass whose collide-stream kernel is queued and whose link
+    // kernel is not yet (lead_src < 0: none): it goes out beside the next
+    // collide-stream kernel, or when the queue ends.  lead_steps: its steps.
+    int lead_src = -1, lead_pre = 0, lead_steps = 1;
+    // Multi-step passes (lbm_march.cu): whether the grid takes them, their
+    // plan, and the intermediate states near the body, one set per source
+    // buffer, allocated at first use.
+    bool march = false;
+    alignas(64) CUtensorMap pmap[NBUF];  // one-row boxes of the population buffers
+    MarchPlan plan;
+    int bounce[4] = {1, 0, 1, 0}, keep[4] = {1, 0, 1, 0};
+    int2 *march_units_d = nullptr;  // the work of each CTA of a pass
+    int n_units = 0;
+    char *mid = nullptr;          // [NBUF][GROUP_STEPS - 1] states of the kept rows
+    double *group_partials = nullptr;  // [GROUP_STEPS] slices of control-volume rows
+    long long *front = nullptr;   // steps done by the collide-stream kernels, on the device
+    long long front_host = -1;    // its value once the queued work is done
     int link_prio = 0;           // launch priority of the link kernels (the device's highest)
     double adj_budget = 0;       // bytes the adjoint may fill with kept states (0: from free memory)
     uint8_t *mask_d = nullptr;
@@ -89,6 +109,7 @@ struct lbm_ctx {
     void *inlet = nullptr;
     double *partials = nullptr;  // NBUF slices, one per destination buffer
     double *link_partials = nullptr;
+    double *link_totals = nullptr;  // behind link_partials, one allocation
     unsigned int *ticket = nullptr;
     int link_ctas = 1;
     double link_base[2] = {0, 0}, flux_base[2] = {0, 0};
@@ -106,6 +127,8 @@ struct lbm_ctx {
     long long drtt_ready = 0;    // DRTT(s) is final for s < drtt_ready
     // [start buffer][GRAPH_STEPS or NBUF steps][opens with the previous step's link kernel]
     cudaGraphExec_t graph[NBUF][2][2] = {};
+    // [start buffer][GRAPH_PASSES[k] passes][opens with the previous pass's link kernel]
+    cudaGraphExec_t pass_graph[NBUF][2][2] = {};
     bool timing = false;
     std::vector<cudaEvent_t> events;
     double kt_ms[2] = {0, 0};
@@ -182,10 +205,9 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
     return fn;
 }
 
-// Tensor map over one population buffer viewed as [9][ny][pitch], with the
-// staged kernel's box: 128 + 2 PAD columns (PAD = 16 bytes of elements), the
-// tile rows plus one above and one below, all nine planes.
-bool encode_tensor_map(CUtensorMap *m, int storage, void *base, int pitch, int ny)
+// Tensor map over one population buffer viewed as [9][ny][pitch], with a box
+// of `columns` x `rows` of all nine planes.
+bool encode_tensor_map(CUtensorMap *m, int storage, void *base, int pitch, int ny, int columns, int rows)
 {
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (!enc) return false;
@@ -195,8 +217,7 @@ bool encode_tensor_map(CUtensorMap *m, int storage, void *base, int pitch, int n
                                                             : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     const cuuint64_t dims[3] = {(cuuint64_t)pitch, (cuuint64_t)ny, 9};
     const cuuint64_t strides[2] = {(cuuint64_t)pitch * elem, (cuuint64_t)pitch * ny * elem};
-    const cuuint32_t box[3] = {(cuuint32_t)(TILE_X + 2 * (16 / elem)),
-                               (cuuint32_t)(tile_rows(storage) + 2), 9};
+    const cuuint32_t box[3] = {(cuuint32_t)columns, (cuuint32_t)rows, 9};
     const cuuint32_t estr[3] = {1, 1, 1};
     return enc(m, dt, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -262,7 +283,7 @@ LinkArgs link_args(lbm_ctx *h, int src, int dst, int precollision, int drtt_only
     a.status = h->status;
     a.carry = h->carry;
     a.step_ctr = h->step_ctr;
-    a.plane = h->plane;
+    a.plane = a.dst_plane = h->plane;
     a.nx = h->nx;
     a.ny = h->ny;
     a.pitch = h->pitch;
@@ -278,16 +299,86 @@ LinkArgs link_args(lbm_ctx *h, int src, int dst, int precollision, int drtt_only
     return a;
 }
 
-// The link kernel of the step that read buffer src, on the side stream,
-// forked after everything queued so far on the handle's stream (that step's
-// collide-stream kernel included); the collide-stream kernel that overwrites
-// src next waits for it (ev_read).
-cudaError_t launch_link_side(lbm_ctx *h, int src, int precollision)
+// The link kernel's arguments for one step from buffer src.
+LinkGroupArgs link_group(lbm_ctx *h, const LinkArgs &a)
 {
-    LinkArgs la = link_args(h, src, next_buf(src), precollision, 0);
+    LinkGroupArgs g;
+    memset(&g, 0, sizeof(g));
+    g.a = a;
+    g.steps = 1;
+    g.state[0] = a.src;
+    g.state[1] = a.dst;
+    g.plane[0] = g.plane[1] = h->plane;
+    g.partials[0] = a.partials;
+    g.totals = h->link_totals;
+    return g;
+}
+
+// Elements between two planes of an intermediate state (the kept rows).
+long long mid_plane(const lbm_ctx *h) { return (long long)(h->keep[3] - h->keep[2] + 1) * h->pitch; }
+
+// First element of intermediate state j of the pass from buffer src.
+char *mid_state(const lbm_ctx *h, int src, int j)
+{
+    return h->mid + ((size_t)src * (GROUP_STEPS - 1) + j) * 9 * (size_t)mid_plane(h) * h->elem;
+}
+
+// The states of the pass from buffer src, t .. t + GROUP_STEPS, addressed by
+// grid row: the intermediate ones hold the kept rows only.
+void pass_states(const lbm_ctx *h, int src, const void **state, long long *plane)
+{
+    for (int j = 0; j <= GROUP_STEPS; ++j) {
+        if (j == 0 || j == GROUP_STEPS) {
+            state[j] = h->pop[j == 0 ? src : next_buf(src)];
+            plane[j] = h->plane;
+        } else {
+            state[j] = mid_state(h, src, j - 1) - (long long)h->keep[2] * h->pitch * (long long)h->elem;
+            plane[j] = mid_plane(h);
+        }
+    }
+}
+
+MarchArgs march_args(lbm_ctx *h, int src)
+{
+    MarchArgs m;
+    memset(&m, 0, sizeof(m));
+    m.s = step_args(h, src, next_buf(src), 0);
+    for (int j = 0; j + 1 < GROUP_STEPS; ++j) m.mid[j] = mid_state(h, src, j);
+    m.mid_plane = mid_plane(h);
+    m.out_w = h->plan.out_w;
+    m.units = h->march_units_d;
+    m.n_units = h->n_units;
+    memcpy(m.bounce, h->bounce, sizeof(m.bounce));
+    memcpy(m.keep, h->keep, sizeof(m.keep));
+    m.front = h->front;
+    m.ticket = h->ticket + 8;
+    return m;
+}
+
+// The link kernel of the step (or, after the control-volume sums, of the
+// pass) that read buffer src, on the side stream, forked after everything
+// queued so far on the handle's stream (its collide-stream kernel included);
+// the collide-stream kernel that overwrites src next waits for it (ev_read).
+cudaError_t launch_link_side(lbm_ctx *h, int src, int precollision, int steps)
+{
+    LinkGroupArgs g = link_group(h, link_args(h, src, next_buf(src), precollision, 0));
     cudaError_t e = cudaEventRecord(h->ev_fork, h->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->ev_fork, 0);
-    if (e == cudaSuccess) e = launch_link_force(h->storage, la, h->side, h->link_prio);
+    if (steps > 1) {
+        CvArgs c;
+        memset(&c, 0, sizeof(c));
+        c.s = step_args(h, src, next_buf(src), 0);
+        pass_states(h, src, c.state, c.plane);
+        pass_states(h, src, g.state, g.plane);
+        g.steps = steps;
+        for (int j = 0; j < steps; ++j) {
+            c.partials[j] = h->group_partials + (size_t)j * CV_PARTIAL * h->n_cv_tiles;
+            g.partials[j] = c.partials[j];
+        }
+        if (e == cudaSuccess) e = launch_cv_sums(h->storage, c, h->side, h->link_prio);
+        h->launches += 1;
+    }
+    if (e == cudaSuccess) e = launch_link_force(h->storage, g, h->side, h->link_prio);
     if (e == cudaSuccess) e = cudaEventRecord(h->ev_read[src], h->side);
     h->ev_live[src] = true;
     h->launches += 1;
@@ -300,7 +391,7 @@ cudaError_t flush_link(lbm_ctx *h)
     if (h->lead_src < 0) return cudaSuccess;
     const int src = h->lead_src;
     h->lead_src = -1;
-    return launch_link_side(h, src, h->lead_pre);
+    return launch_link_side(h, src, h->lead_pre, h->lead_steps);
 }
 
 // Join the side stream back into the handle's stream.
@@ -337,7 +428,7 @@ cudaError_t launch_one_step(lbm_ctx *h, int src, int precollision, cudaEvent_t *
         if (e != cudaSuccess) return e;
         LinkArgs la = link_args(h, src, dst, precollision, 0);
         cudaEventRecord(ev[1], h->stream);
-        e = launch_link_force(h->storage, la, h->stream);
+        e = launch_link_force(h->storage, link_group(h, la), h->stream);
         cudaEventRecord(ev[2], h->stream);
         h->launches += 2;
         return e;
@@ -349,6 +440,23 @@ cudaError_t launch_one_step(lbm_ctx *h, int src, int precollision, cudaEvent_t *
                               h->tmap_ok ? (const void *)&h->tmap[src] : nullptr, h->stream);
     h->lead_src = src;
     h->lead_pre = precollision;
+    h->lead_steps = 1;
+    h->launches += 1;
+    return e;
+}
+
+// One pass t -> t + GROUP_STEPS from buffer src into next_buf(src), its link
+// kernel held as a step's is.
+cudaError_t launch_one_pass(lbm_ctx *h, int src)
+{
+    const int dst = next_buf(src);
+    cudaError_t e = flush_link(h);
+    if (e == cudaSuccess && h->ev_live[dst]) e = cudaStreamWaitEvent(h->stream, h->ev_read[dst], 0);
+    if (e != cudaSuccess) return e;
+    e = launch_march(h->storage, march_args(h, src), &h->pmap[src], h->stream);
+    h->lead_src = src;
+    h->lead_pre = 0;
+    h->lead_steps = GROUP_STEPS;
     h->launches += 1;
     return e;
 }
@@ -362,39 +470,50 @@ void drop_graphs(lbm_ctx *h)
                     cudaGraphExecDestroy(h->graph[p][k][l]);
                     h->graph[p][k][l] = nullptr;
                 }
+    for (int p = 0; p < NBUF; ++p)
+        for (int k = 0; k < 2; ++k)
+            for (int l = 0; l < 2; ++l)
+                if (h->pass_graph[p][k][l]) {
+                    cudaGraphExecDestroy(h->pass_graph[p][k][l]);
+                    h->pass_graph[p][k][l] = nullptr;
+                }
 }
 
-// Captures GRAPH_STEPS (k = 0) or NBUF (k = 1) steps from buffer p.  lead = 1:
-// the graph opens with the held link kernel of the step before (which read
-// prev_buf(p)) beside its first collide-stream kernel.  Either way the graph
-// ends with its last step's link kernel held: the caller sets lead_src.
-lbm_status build_graph(lbm_ctx *h, int p, int k, int lead)
+// Captures GRAPH_STEPS (k = 0) or NBUF (k = 1) steps, or GRAPH_PASSES[k]
+// passes, from buffer p.  lead = 1: the graph opens with the held link kernel
+// of the step or pass before (which read prev_buf(p)) beside its first
+// collide-stream kernel.  Either way the graph ends with its last link kernel
+// held: the caller sets lead_src.
+lbm_status build_graph(lbm_ctx *h, int p, int k, int lead, bool passes)
 {
-    int steps = k == 0 ? GRAPH_STEPS : NBUF;
+    const int units = passes ? GRAPH_PASSES[k] : (k == 0 ? GRAPH_STEPS : NBUF);
     cudaGraph_t g = nullptr;
     for (int b = 0; b < NBUF; ++b) h->ev_live[b] = false;
-    const int saved_src = h->lead_src, saved_pre = h->lead_pre;
+    const int saved_src = h->lead_src, saved_pre = h->lead_pre, saved_steps = h->lead_steps;
     h->lead_src = lead ? prev_buf(p) : -1;
     h->lead_pre = 0;
+    h->lead_steps = passes ? GROUP_STEPS : 1;
     CK(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
     cudaError_t le = cudaSuccess;
     long long saved = h->launches;
     int b = p;
-    for (int s = 0; s < steps && le == cudaSuccess; ++s) {
-        le = launch_one_step(h, b, 0, nullptr);
+    for (int s = 0; s < units && le == cudaSuccess; ++s) {
+        le = passes ? launch_one_pass(h, b) : launch_one_step(h, b, 0, nullptr);
         b = next_buf(b);
     }
     if (le == cudaSuccess) le = join_side(h);
     h->launches = saved;
     h->lead_src = saved_src;
     h->lead_pre = saved_pre;
+    h->lead_steps = saved_steps;
     cudaError_t ee = cudaStreamEndCapture(h->stream, &g);
     if (le != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
         return cuda_err(h, le, "capture step kernels");
     }
     if (ee != cudaSuccess) return cuda_err(h, ee, "end capture");
-    cudaError_t ie = cudaGraphInstantiateWithFlags(&h->graph[p][k][lead], g, cudaGraphInstantiateFlagUseNodePriority);
+    cudaError_t ie = cudaGraphInstantiateWithFlags(passes ? &h->pass_graph[p][k][lead] : &h->graph[p][k][lead], g,
+                                                   cudaGraphInstantiateFlagUseNodePriority);
     cudaGraphDestroy(g);
     if (ie != cudaSuccess) return cuda_err(h, ie, "instantiate graph");
     return LBM_OK;
@@ -419,6 +538,79 @@ lbm_status ensure_series(lbm_ctx *h, long long need)
     h->series_cap = cap;
     drop_graphs(h);
     return LBM_OK;
+}
+
+// Decides whether the grid takes multi-step passes and lays out the rectangles
+// they treat apart, from the solid nodes' bounding box:
+//   bounce: one node wider, which holds every node with a solid neighbour;
+//   keep:   where the link kernel and the control-volume sums read states:
+//           one node wider than that and than the box (pulled neighbours).
+// A rectangle that touches the top or bottom edge covers all rows (y wraps).
+void plan_passes(lbm_ctx *h, const std::vector<long long> &solids)
+{
+    h->march = false;
+    if (h->periodic || !march_grid(h->storage, h->nx, h->ny)) return;
+    int x0 = h->nx, x1 = -1, y0 = h->ny, y1 = -1;
+    for (long long n : solids) {
+        const int x = (int)(n % h->nx), y = (int)(n / h->nx);
+        x0 = x < x0 ? x : x0;
+        x1 = x > x1 ? x : x1;
+        y0 = y < y0 ? y : y0;
+        y1 = y > y1 ? y : y1;
+    }
+    int k[4] = {h->cv[0] - 1, h->cv[1] + 1, h->cv[2] - 1, h->cv[3] + 1};
+    if (x1 >= 0) {
+        h->bounce[0] = x0 - 1;  // solid columns lie in [2, nx - 3]
+        h->bounce[1] = x1 + 1;
+        h->bounce[2] = y0 - 1;
+        h->bounce[3] = y1 + 1;
+        if (h->bounce[2] <= 0 || h->bounce[3] >= h->ny - 1) {
+            h->bounce[2] = 0;
+            h->bounce[3] = h->ny - 1;
+        }
+        k[0] = h->bounce[0] - 1 < k[0] ? h->bounce[0] - 1 : k[0];
+        k[1] = h->bounce[1] + 1 > k[1] ? h->bounce[1] + 1 : k[1];
+        k[2] = h->bounce[2] - 1 < k[2] ? h->bounce[2] - 1 : k[2];
+        k[3] = h->bounce[3] + 1 > k[3] ? h->bounce[3] + 1 : k[3];
+    }
+    if (k[0] < 0) k[0] = 0;
+    if (k[1] > h->nx - 1) k[1] = h->nx - 1;
+    if (k[2] <= 0 || k[3] >= h->ny - 1) {
+        k[2] = 0;
+        k[3] = h->ny - 1;
+    }
+    memcpy(h->keep, k, sizeof(k));
+    if ((double)(k[1] - k[0] + 1) * (k[3] - k[2] + 1) > MARCH_KEEP_SHARE * h->nx * h->ny) return;
+    h->march = true;
+}
+
+// The buffers of the multi-step passes, at first use.  Without room for them
+// the handle takes single steps.
+void ensure_passes(lbm_ctx *h)
+{
+    if (!h->march || h->mid) return;
+    const size_t state = 9 * (size_t)mid_plane(h) * h->elem;
+    h->mid = (char *)dev_alloc(h, state * NBUF * (GROUP_STEPS - 1));
+    h->group_partials = (double *)dev_alloc(h, sizeof(double) * GROUP_STEPS * CV_PARTIAL * h->n_cv_tiles);
+    std::vector<int2> units;
+    h->plan = march_plan(h->storage, h->nx, h->ny, h->sm_count, h->bounce, h->keep, &units);
+    h->n_units = (int)units.size();
+    h->march_units_d = (int2 *)dev_alloc(h, sizeof(int2) * units.size());
+    bool ok = h->mid && h->group_partials && h->march_units_d;
+    ok = ok && cudaMemcpyAsync(h->march_units_d, units.data(), sizeof(int2) * units.size(), cudaMemcpyHostToDevice,
+                               h->stream) == cudaSuccess &&
+         cudaStreamSynchronize(h->stream) == cudaSuccess;
+    for (int b = 0; b < NBUF; ++b)
+        ok = ok && encode_tensor_map(&h->pmap[b], h->storage, h->pop[b], h->pitch, h->ny, march_box_columns(h->storage), 1);
+    if (!ok) {
+        dev_free(h, h->mid);
+        dev_free(h, h->group_partials);
+        dev_free(h, h->march_units_d);
+        h->mid = nullptr;
+        h->group_partials = nullptr;
+        h->march_units_d = nullptr;
+        h->march = false;
+    }
 }
 
 lbm_status flush_timing(lbm_ctx *h, int nev)
@@ -453,7 +645,7 @@ lbm_status finalize_drtt(lbm_ctx *h)
                                 true, nullptr, h->stream),
        "momentum pass");
     LinkArgs la = link_args(h, h->cur, slot, 0, 1);
-    CK(h, launch_link_force(h->storage, la, h->stream), "DRTT finalize");
+    CK(h, launch_link_force(h->storage, link_group(h, la), h->stream), "DRTT finalize");
     h->launches += 2;
     h->drtt_ready = h->t;
     return LBM_OK;
@@ -471,7 +663,7 @@ void free_all(lbm_ctx *h)
     void *bufs[] = {h->pop_base[0], h->pop_base[1], h->pop_base[2], h->mask_d, h->nbits, h->tile_flag, h->links,
                     h->bnodes,
                     h->u_row, h->inlet, h->partials, h->link_partials, h->ticket, h->series,
-                    h->carry, h->step_ctr, h->status};
+                    h->carry, h->step_ctr, h->status, h->mid, h->group_partials, h->march_units_d};
     for (void *p : bufs) dev_free(h, p);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
@@ -513,9 +705,11 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
     if ((bc.alloc == nullptr) != (bc.free == nullptr))
         return set_err(nullptr, LBM_EINVAL, "alloc and free must be given together");
     const int periodic = bc.kind == LBM_BC_PERIODIC;
-    // the mask's solid nodes, scanned once for the default box and the base sums
+    // the mask's solid nodes, scanned once for the default box, the base sums
+    // and the passes' rectangles
     std::vector<long long> solids;
-    const bool need_solids = bc.cv[0] < 0 || bc.storage == LBM_F32_DEV || bc.storage == LBM_F16_DEV;
+    const bool need_solids = bc.cv[0] < 0 || bc.storage == LBM_F32_DEV || bc.storage == LBM_F16_DEV ||
+                             (!periodic && march_grid(bc.storage, nx, ny));
     if (mask && need_solids && nx > 0 && ny > 0 && (long long)nx * ny * 8 < (1LL << 31))
         solids = solid_nodes(mask, nx, ny);
     int cv[4];
@@ -624,7 +818,10 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
     if (h->use_bulk) {
         h->tmap_ok = true;
         for (int b = 0; b < NBUF; ++b)
-            h->tmap_ok = h->tmap_ok && encode_tensor_map(&h->tmap[b], h->storage, h->pop[b], h->pitch, ny);
+            h->tmap_ok = h->tmap_ok &&
+                         // the staged kernel's box: a tile with 16 bytes of columns and one row more on each side
+                         encode_tensor_map(&h->tmap[b], h->storage, h->pop[b], h->pitch, ny,
+                                           TILE_X + 2 * (16 / (int)h->elem), tile_rows(h->storage) + 2);
         if (!h->tmap_ok)
             return fail(set_err(h, LBM_ECUDA, "tensor maps for the staged kernel could not be encoded"));
     }
@@ -634,10 +831,13 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
     ALLOC(h->u_row, double *, sizeof(double) * ny);
     ALLOC(h->inlet, void *, 9 * (size_t)ny * h->elem);
     ALLOC(h->partials, double *, sizeof(double) * NBUF * CV_PARTIAL * h->n_cv_tiles);
-    ALLOC(h->link_partials, double *, sizeof(double) * LINK_PARTIAL * MAX_LINK_CTAS * LINK_WARPS);
-    ALLOC(h->ticket, unsigned int *, sizeof(unsigned int));
+    const size_t link_rows = (size_t)GROUP_STEPS * LINK_PARTIAL * MAX_LINK_CTAS * LINK_WARPS;
+    ALLOC(h->link_partials, double *, sizeof(double) * (link_rows + 16 * GROUP_STEPS));
+    h->link_totals = h->link_partials + link_rows;
+    ALLOC(h->ticket, unsigned int *, sizeof(unsigned int) * 16);
     ALLOC(h->carry, double *, sizeof(double) * 8);
-    ALLOC(h->step_ctr, long long *, sizeof(long long));
+    ALLOC(h->step_ctr, long long *, sizeof(long long) * 2);
+    h->front = h->step_ctr + 1;
     ALLOC(h->status, int *, sizeof(int) * 2);
     st = ensure_series(h, 1024);
     if (st != LBM_OK) return fail(st);
@@ -649,9 +849,9 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
         CKC(cudaMemsetAsync(h->pop_base[b], 0, guard_front + pop_bytes + guard_back, s), "memset");
     CKC(cudaMemsetAsync(h->nbits, 0, sizeof(uint16_t) * h->plane, s), "memset");
     CKC(cudaMemsetAsync(h->partials, 0, sizeof(double) * NBUF * CV_PARTIAL * h->n_cv_tiles, s), "memset");
-    CKC(cudaMemsetAsync(h->ticket, 0, sizeof(unsigned int), s), "memset");
+    CKC(cudaMemsetAsync(h->ticket, 0, sizeof(unsigned int) * 16, s), "memset");
     CKC(cudaMemsetAsync(h->carry, 0, sizeof(double) * 8, s), "memset");
-    CKC(cudaMemsetAsync(h->step_ctr, 0, sizeof(long long), s), "memset");
+    CKC(cudaMemsetAsync(h->step_ctr, 0, sizeof(long long) * 2, s), "memset");
     const int status0[2] = {0, INT_MAX};
     CKC(cudaMemcpyAsync(h->status, status0, sizeof(status0), cudaMemcpyHostToDevice, s), "H2D status");
     h->status_armed = true;
@@ -697,6 +897,7 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
             h->first_r0 = r0;
             h->first_r1 = r1;
         }
+        plan_passes(h, solids);
         h->nlinks = total;
         {
             long long work = total > h->n_cv_tiles ? total : h->n_cv_tiles;
@@ -764,10 +965,18 @@ lbm_status queue_steps(lbm_ctx *h, int n)
             if (!e) CK(h, cudaEventCreate(&e), "event create");
     }
     int nev = 0;
+    if (n >= GROUP_STEPS) ensure_passes(h);
     while (n > 0) {
-        if (h->precollision || h->timing || n < NBUF) {
+        const bool marching = h->march && !h->use_bulk && !h->timing;
+        const bool pass = marching && !h->precollision && n >= GROUP_STEPS;
+        if (pass && h->front_host != h->t) {
+            CK(h, launch_set_front(h->front, h->t, h->stream), "step counter");
+            h->front_host = h->t;
+            h->launches += 1;
+        }
+        if (pass ? n < NBUF * GROUP_STEPS : (h->precollision || h->timing || n < NBUF || marching)) {
             cudaEvent_t *ev = h->timing ? &h->events[3 * nev] : nullptr;
-            CK(h, launch_one_step(h, h->cur, h->precollision, ev), "step launch");
+            CK(h, pass ? launch_one_pass(h, h->cur) : launch_one_step(h, h->cur, h->precollision, ev), "step launch");
             if (h->timing && ++nev == TIMING_BATCH) {
                 st = flush_timing(h, nev);
                 if (st != LBM_OK) return st;
@@ -775,26 +984,31 @@ lbm_status queue_steps(lbm_ctx *h, int n)
             }
             h->cur = next_buf(h->cur);
             h->precollision = 0;
-            h->t += 1;
-            n -= 1;
+            h->t += pass ? GROUP_STEPS : 1;
+            n -= pass ? GROUP_STEPS : 1;
+            if (pass) h->front_host += GROUP_STEPS;
         } else {
-            int k = n >= GRAPH_STEPS ? 0 : 1;
-            int steps = k == 0 ? GRAPH_STEPS : NBUF;
-            // a held link kernel of the step before opens the graph
-            const int lead = h->lead_src == prev_buf(h->cur) && !h->lead_pre ? 1 : 0;
+            const int each = pass ? GROUP_STEPS : 1;
+            const int k = n >= each * (pass ? GRAPH_PASSES[0] : GRAPH_STEPS) ? 0 : 1;
+            const int units = pass ? GRAPH_PASSES[k] : (k == 0 ? GRAPH_STEPS : NBUF);
+            // a held link kernel of the step or pass before opens the graph
+            const int lead = h->lead_src == prev_buf(h->cur) && !h->lead_pre && h->lead_steps == each ? 1 : 0;
             if (!lead) CK(h, flush_link(h), "link launch");
             // the graph's first steps overwrite buffers that launched link kernels read
             CK(h, join_side(h), "join");
-            if (!h->graph[h->cur][k][lead]) {
-                st = build_graph(h, h->cur, k, lead);
+            cudaGraphExec_t *g = pass ? &h->pass_graph[h->cur][k][lead] : &h->graph[h->cur][k][lead];
+            if (!*g) {
+                st = build_graph(h, h->cur, k, lead, pass);
                 if (st != LBM_OK) return st;
             }
-            CK(h, cudaGraphLaunch(h->graph[h->cur][k][lead], h->stream), "graph launch");
-            h->lead_src = prev_buf(h->cur);  // steps is a multiple of NBUF
+            CK(h, cudaGraphLaunch(*g, h->stream), "graph launch");
+            h->lead_src = prev_buf(h->cur);  // units is a multiple of NBUF
             h->lead_pre = 0;
-            h->launches += 2 * steps - 1 + lead;  // the last link kernel is held
-            h->t += steps;
-            n -= steps;
+            h->lead_steps = each;
+            h->launches += (pass ? 3 : 2) * (long long)units - (pass ? 2 : 1) * (1 - lead);  // the last link kernel is held
+            h->t += (long long)units * each;
+            if (pass) h->front_host += (long long)units * each;
+            n -= units * each;
         }
     }
     CK(h, flush_link(h), "link launch");
@@ -972,11 +1186,13 @@ lbm_status lbm_prepare(lbm_ctx *h, long n)
     if (n < 0) return set_err(h, LBM_EINVAL, "n must be >= 0");
     lbm_status st = ensure_series(h, h->t + n);
     if (st != LBM_OK) return st;
+    ensure_passes(h);
+    const bool pass = h->march && !h->use_bulk;  // such a handle replays no graph of single steps
     for (int p = 0; p < NBUF; ++p)
         for (int k = 0; k < 2; ++k)
             for (int l = 0; l < 2; ++l)
-                if (!h->graph[p][k][l]) {
-                    st = build_graph(h, p, k, l);
+                if (!(pass ? h->pass_graph : h->graph)[p][k][l]) {
+                    st = build_graph(h, p, k, l, pass);
                     if (st != LBM_OK) return st;
                 }
     return LBM_OK;

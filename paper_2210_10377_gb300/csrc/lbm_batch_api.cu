@@ -253,6 +253,7 @@ LinkArgs link_args(const lbm_batch *b, int d, int s, int src)
     a.carry = b->carry + 8 * d;
     a.step_ctr = b->step_ctr;
     a.plane = m.plane;
+    a.dst_plane = m.plane;
     a.nx = m.nx;
     a.ny = m.ny;
     a.pitch = m.pitch;

@@ -15,10 +15,11 @@
 //   partials     [3][n_cv_tiles][6] (one slice per destination buffer) per-tile J(t) on the pre- and on the
 //                post-collision state, and gained-minus-lost(t); FP64 for FP64
 //                storage, float-float pairs otherwise (8 bytes either way);
-//   link_partials [n_ctas][12] per-CTA rows of the link kernel, same types;
+//   link_partials [GROUP_STEPS][warps][14] per-warp rows of the link kernel, same types;
 //   series       double [steps][12]: A, B, DRTT, A', momentum defect, SI (x, y each);
 //   carry        double [8]: J_post(t-1), GL(t-1), flag;  step counter int64;
-//   ticket       uint32 arrival counter of the link kernel's CTAs.
+//   ticket       uint32 arrival counters: of the link kernel's warps (one per
+//                step of a launch, one for the steps) and of the multi-step kernel.
 #pragma once
 
 #include <cuda.h>
@@ -48,6 +49,8 @@ constexpr int MAX_LINK_CTAS = 148;
 constexpr int CV_PARTIAL = 6;
 constexpr int LINK_PARTIAL = 14;
 constexpr int SERIES_ROW = 12;
+// Steps of one multi-step pass (lbm_march.cu) and of one link-kernel launch at most.
+constexpr int GROUP_STEPS = 4;
 
 // Tile rows of the FP32 and FP16-deviation kernels (tuning knobs).
 #ifndef GBLBM_TR_F16
@@ -187,6 +190,19 @@ struct LinkArgs {
     float visc_f;
     double link_base[2];     // deviation storage: 2 rho0 sum_links c_i w_i
     double flux_base[2];     // deviation storage: rho0 (sum_in - sum_out) c_i w_i
+    long long dst_plane;     // elements per plane of dst (plane: of src)
+};
+
+// One launch of the link kernel over `steps` consecutive steps: step j reads
+// state[j] and state[j + 1] (a.src, a.dst, a.plane, a.dst_plane and
+// a.partials are set from these per step).
+struct LinkGroupArgs {
+    LinkArgs a;
+    int steps;
+    const void *state[GROUP_STEPS + 1];
+    long long plane[GROUP_STEPS + 1];
+    const double *partials[GROUP_STEPS];
+    double *totals;          // [GROUP_STEPS][16]: the reduced sums of each step
 };
 
 // Message returned by lbm_last_error(NULL) on the calling thread.
@@ -226,7 +242,7 @@ size_t tma_stage_bytes(int storage);
 int collide_stream_prefetch_rows(int storage, int sm_count, int tiles_x);
 // priority: the launch's scheduling priority (0: the stream's own; lower
 // numbers are served first)
-cudaError_t launch_link_force(int storage, const LinkArgs &a, cudaStream_t st, int priority = 0);
+cudaError_t launch_link_force(int storage, const LinkGroupArgs &g, cudaStream_t st, int priority = 0);
 cudaError_t launch_gather(int storage, const void *pop, const uint16_t *nbits, const void *inlet,
                           long long plane, int nx, int ny, int pitch, int periodic,
                           int precollision, double rho0, int plane_i, double *out,

@@ -80,7 +80,7 @@ __device__ __forceinline__ void link_sums(const LinkArgs &a, long long k0, long 
             // f_opp(i)(x_f, t): x_f + c_i is solid, so it is the bounced ft_i(x_f, t-1)
             fo = to_comp(src[i * plane + idx]);
         }
-        const T ft = to_comp(dst[i * plane + idx]);
+        const T ft = to_comp(dst[i * a.dst_plane + idx]);
         A sa, sb, sp;
         if constexpr (S == LBM_F64) {
             sa = fi + fo;
@@ -220,12 +220,25 @@ __device__ __forceinline__ void finish_rows_warp(const LinkArgs &a, double dk, l
 #ifndef GBLBM_LINK_EARLY
 #define GBLBM_LINK_EARLY 1
 #endif
-template <int S>
-__global__ void __launch_bounds__(LINK_THREADS) k_link_force(LinkArgs a)
+// GROUP: the launch covers several steps (blockIdx.y); each step's last warp
+// leaves its totals in g.totals, and the last of those warps completes the
+// rows of all steps in order.
+template <int S, bool GROUP>
+__global__ void __launch_bounds__(LINK_THREADS) k_link_force(const __grid_constant__ LinkGroupArgs g)
 {
     using A = typename AccOf<S>::type;
+    const int step = GROUP ? blockIdx.y : 0;
+    const LinkArgs &a = g.a;
     A v[LINK_PARTIAL];
     {
+        LinkArgs l = g.a;
+        if constexpr (GROUP) {
+            l.src = g.state[step];
+            l.dst = g.state[step + 1];
+            l.plane = g.plane[step];
+            l.dst_plane = g.plane[step + 1];
+            l.partials = g.partials[step];
+        }
         const long long nl = a.drtt_only ? 0 : a.nlinks;
         const long long per = (nl + gridDim.x - 1) / gridDim.x;
         const long long k0 = per * blockIdx.x;
@@ -233,23 +246,24 @@ __global__ void __launch_bounds__(LINK_THREADS) k_link_force(LinkArgs a)
         const int per_p = (a.n_partials + gridDim.x - 1) / gridDim.x;
         const int p0 = per_p * blockIdx.x;
         const int p1 = p0 + per_p < a.n_partials ? p0 + per_p : a.n_partials;
-        link_sums<S, LINK_THREADS, GBLBM_LINK_EARLY != 0>(a, k0, k1 > k0 ? k1 : k0, p0, p1 > p0 ? p1 : p0, v);
+        link_sums<S, LINK_THREADS, GBLBM_LINK_EARLY != 0>(l, k0, k1 > k0 ? k1 : k0, p0, p1 > p0 ? p1 : p0, v);
     }
     // each warp reduces its sums and writes them as one row (slot: CTA, warp);
-    // no block barrier, and the last warp to take a ticket completes the step
+    // no block barrier, and the last warp of a step to take a ticket sums it
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1)
 #pragma unroll
         for (int k = 0; k < LINK_PARTIAL; ++k) acc_add(v[k], shfl_down(v[k], d));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rows = (int)gridDim.x * LINK_WARPS;
+    A *const all = (A *)a.link_partials + (long long)LINK_PARTIAL * rows * step;
     unsigned int ticket = 0;
     if (lane == 0) {
-        A *row = (A *)a.link_partials + LINK_PARTIAL * ((long long)blockIdx.x * LINK_WARPS + warp);
+        A *row = all + LINK_PARTIAL * ((long long)blockIdx.x * LINK_WARPS + warp);
 #pragma unroll
         for (int k = 0; k < LINK_PARTIAL; ++k) row[k] = v[k];
         __threadfence();
-        ticket = atomicAdd(a.ticket, 1u);
+        ticket = atomicAdd(a.ticket + step, 1u);
     }
     ticket = __shfl_sync(0xffffffffu, ticket, 0);
     if (ticket != (unsigned int)rows - 1) return;
@@ -264,7 +278,7 @@ __global__ void __launch_bounds__(LINK_THREADS) k_link_force(LinkArgs a)
     A mine;
     acc_zero(mine);
     if (k < LINK_PARTIAL) {
-        const A *col = (const A *)a.link_partials + k;
+        const A *col = all + k;
         for (int b = r0; b < r1; ++b) {
             A r;
             if constexpr (S == LBM_F64)
@@ -278,36 +292,51 @@ __global__ void __launch_bounds__(LINK_THREADS) k_link_force(LinkArgs a)
         const A upper = shfl_down(mine, 16);
         if (lane < 16) acc_add(mine, upper);
     }
-    const double dk = acc_double(mine);
-    const long long t = *a.step_ctr;
-    // Series slot of a step: the step itself, or its parity when only the
-    // last two rows are kept.  A slot beyond the buffer (an internal
-    // invariant: the host grows the series before every launch) is not
-    // written and raises status bit 4.
-    const bool keep_all = a.record_series != 0;
-    const long long kp = keep_all ? t - 1 : ((t - 1) & 1), kc = keep_all ? t : (t & 1);
-    double *prev = nullptr, *cur = nullptr;
-    if (t >= 1 && a.carry[4] != 0.0) {
-        if (kp < a.series_rows)
-            prev = a.series + SERIES_ROW * kp;
-        else if (lane == 0)
-            atomicOr(a.status, 4);
+    double dk = acc_double(mine);
+    if (lane == 0) a.ticket[step] = 0u;
+    // the last step's warp to arrive completes the rows of all steps in order
+    if constexpr (GROUP) {
+        if (lane < 16) __stcg(g.totals + 16 * step + lane, dk);
+        __threadfence();
+        __syncwarp();
+        unsigned int last = 0;
+        if (lane == 0) last = atomicAdd(a.ticket + GROUP_STEPS, 1u);
+        last = __shfl_sync(0xffffffffu, last, 0);
+        if (last != (unsigned int)g.steps - 1) return;
+        __threadfence();
+        if (lane == 0) a.ticket[GROUP_STEPS] = 0u;
     }
-    if (!a.drtt_only) {
-        if (kc < a.series_rows)
-            cur = a.series + SERIES_ROW * kc;
-        else if (lane == 0)
-            atomicOr(a.status, 4);
+    const long long t0 = *a.step_ctr;
+    const int steps = GROUP ? g.steps : 1;
+    for (int j = 0; j < steps; ++j) {
+        if constexpr (GROUP) dk = __ldcg(g.totals + 16 * j + (lane & 15));
+        const long long t = t0 + j;
+        // Series slot of a step: the step itself, or its parity when only the
+        // last two rows are kept.  A slot beyond the buffer (an internal
+        // invariant: the host grows the series before every launch) is not
+        // written and raises status bit 4.
+        const bool keep_all = a.record_series != 0;
+        const long long kp = keep_all ? t - 1 : ((t - 1) & 1), kc = keep_all ? t : (t & 1);
+        double *prev = nullptr, *cur = nullptr;
+        if (t >= 1 && a.carry[4] != 0.0) {
+            if (kp < a.series_rows)
+                prev = a.series + SERIES_ROW * kp;
+            else if (lane == 0)
+                atomicOr(a.status, 4);
+        }
+        if (!a.drtt_only) {
+            if (kc < a.series_rows)
+                cur = a.series + SERIES_ROW * kc;
+            else if (lane == 0)
+                atomicOr(a.status, 4);
+        }
+        finish_rows_warp(a, dk, t, prev, cur, a.drtt_only != 0);
+        __syncwarp();
     }
-    finish_rows_warp(a, dk, t, prev, cur, a.drtt_only != 0);
-    __syncwarp();
-    if (lane == 0) {
-        *a.ticket = 0u;
-        if (!a.drtt_only) *a.step_ctr = t + 1;
-    }
+    if (lane == 0 && !a.drtt_only) *a.step_ctr = t0 + steps;
 }
 
-cudaError_t launch_link_force(int storage, const LinkArgs &a, cudaStream_t st, int priority)
+cudaError_t launch_link_force(int storage, const LinkGroupArgs &g, cudaStream_t st, int priority)
 {
     // The priority travels with the launch, so that a captured graph node
     // keeps it: the link kernel runs beside a collide-stream kernel that
@@ -316,17 +345,20 @@ cudaError_t launch_link_force(int storage, const LinkArgs &a, cudaStream_t st, i
     attr[0].id = cudaLaunchAttributePriority;
     attr[0].val.priority = priority;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.n_ctas);
+    cfg.gridDim = dim3(g.a.n_ctas, g.steps);
     cfg.blockDim = dim3(LINK_THREADS);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = priority != 0 ? 1 : 0;
+    const bool group = g.steps > 1;
     switch (storage) {
-    case LBM_F64: return cudaLaunchKernelEx(&cfg, k_link_force<LBM_F64>, a);
-    case LBM_F32: return cudaLaunchKernelEx(&cfg, k_link_force<LBM_F32>, a);
-    case LBM_F32_DEV: return cudaLaunchKernelEx(&cfg, k_link_force<LBM_F32_DEV>, a);
-    default: return cudaLaunchKernelEx(&cfg, k_link_force<LBM_F16_DEV>, a);
+#define GBLBM_LF(S) (group ? cudaLaunchKernelEx(&cfg, k_link_force<S, true>, g) : cudaLaunchKernelEx(&cfg, k_link_force<S, false>, g))
+    case LBM_F64: return GBLBM_LF(LBM_F64);
+    case LBM_F32: return GBLBM_LF(LBM_F32);
+    case LBM_F32_DEV: return GBLBM_LF(LBM_F32_DEV);
+    default: return GBLBM_LF(LBM_F16_DEV);
+#undef GBLBM_LF
     }
 }
 
