@@ -49,6 +49,14 @@ constexpr int GRAPH_PASSES[2] = {12, NBUF};
 // Share of the grid that the kept intermediate states may cover: with more of
 // it the pass writes so much that single steps are as fast.
 constexpr double MARCH_KEEP_SHARE = 0.25;
+// How GROUP_STEPS steps are taken together, with one link kernel for them:
+// by the multi-step kernel; or by single-step launches into buffers of their
+// own, on grids whose single steps are shorter than a link kernel (17 us of
+// latency): one of those a step bounded them (512 x 256 FP32: 10.5 us a step
+// with two link kernels in flight).  The second kind holds nine more states,
+// so it is for states of at most PASS_STATE_BYTES.
+enum PassKind { PASS_NONE = 0, PASS_MARCH, PASS_STEPS };
+constexpr double PASS_STATE_BYTES = 64e6;
 
 }  // namespace
 
@@ -83,19 +91,22 @@ struct lbm_ctx {
     // kernel is not yet (lead_src < 0: none): it goes out beside the next
     // collide-stream kernel, or when the queue ends.  lead_steps: its steps.
     int lead_src = -1, lead_pre = 0, lead_steps = 1;
-    // Multi-step passes (lbm_march.cu): whether the grid takes them, their
-    // plan, and the intermediate states near the body, one set per source
-    // buffer, allocated at first use.
-    bool march = false;
+    // Passes of GROUP_STEPS steps: the kind that the grid takes, the plan of
+    // the multi-step kernel, and the intermediate states (of the rows `keep`),
+    // one set per source buffer, allocated at first use.
+    int pass_kind = PASS_NONE;
     alignas(64) CUtensorMap pmap[NBUF];  // one-row boxes of the population buffers
     MarchPlan plan;
     int bounce[4] = {1, 0, 1, 0}, keep[4] = {1, 0, 1, 0};
     int2 *march_units_d = nullptr;  // the work of each CTA of a pass
     int n_units = 0;
     char *mid = nullptr;          // [NBUF][GROUP_STEPS - 1] states of the kept rows
-    double *group_partials = nullptr;  // [GROUP_STEPS] slices of control-volume rows
-    long long *front = nullptr;   // steps done by the collide-stream kernels, on the device
-    long long front_host = -1;    // its value once the queued work is done
+    double *group_partials = nullptr;  // [NBUF][GROUP_STEPS] slices of control-volume rows
+    // [NBUF] the step at which the pass from each buffer starts, for the
+    // kernels' reports; a pass sets its successor's (the step counter itself
+    // follows the link kernels, which lag behind)
+    long long *front = nullptr;
+    long long front_host = -1;    // the next pass's entry is set for this step
     int link_prio = 0;           // launch priority of the link kernels (the device's highest)
     double adj_budget = 0;       // bytes the adjoint may fill with kept states (0: from free memory)
     uint8_t *mask_d = nullptr;
@@ -338,11 +349,19 @@ void pass_states(const lbm_ctx *h, int src, const void **state, long long *plane
     }
 }
 
+// The control-volume rows of step j of the pass from buffer src.
+double *pass_partials(const lbm_ctx *h, int src, int j)
+{
+    return h->group_partials + ((size_t)src * GROUP_STEPS + j) * CV_PARTIAL * h->n_cv_tiles;
+}
+
 MarchArgs march_args(lbm_ctx *h, int src)
 {
     MarchArgs m;
     memset(&m, 0, sizeof(m));
     m.s = step_args(h, src, next_buf(src), 0);
+    m.s.step_ctr = h->front + src;
+    m.s.next_ctr = h->front + next_buf(src);
     for (int j = 0; j + 1 < GROUP_STEPS; ++j) m.mid[j] = mid_state(h, src, j);
     m.mid_plane = mid_plane(h);
     m.out_w = h->plan.out_w;
@@ -350,8 +369,6 @@ MarchArgs march_args(lbm_ctx *h, int src)
     m.n_units = h->n_units;
     memcpy(m.bounce, h->bounce, sizeof(m.bounce));
     memcpy(m.keep, h->keep, sizeof(m.keep));
-    m.front = h->front;
-    m.ticket = h->ticket + 8;
     return m;
 }
 
@@ -371,12 +388,11 @@ cudaError_t launch_link_side(lbm_ctx *h, int src, int precollision, int steps)
         pass_states(h, src, c.state, c.plane);
         pass_states(h, src, g.state, g.plane);
         g.steps = steps;
-        for (int j = 0; j < steps; ++j) {
-            c.partials[j] = h->group_partials + (size_t)j * CV_PARTIAL * h->n_cv_tiles;
-            g.partials[j] = c.partials[j];
+        for (int j = 0; j < steps; ++j) g.partials[j] = c.partials[j] = pass_partials(h, src, j);
+        if (h->pass_kind == PASS_MARCH) {  // single steps have written their own
+            if (e == cudaSuccess) e = launch_cv_sums(h->storage, c, h->side, h->link_prio);
+            h->launches += 1;
         }
-        if (e == cudaSuccess) e = launch_cv_sums(h->storage, c, h->side, h->link_prio);
-        h->launches += 1;
     }
     if (e == cudaSuccess) e = launch_link_force(h->storage, g, h->side, h->link_prio);
     if (e == cudaSuccess) e = cudaEventRecord(h->ev_read[src], h->side);
@@ -453,11 +469,28 @@ cudaError_t launch_one_pass(lbm_ctx *h, int src)
     cudaError_t e = flush_link(h);
     if (e == cudaSuccess && h->ev_live[dst]) e = cudaStreamWaitEvent(h->stream, h->ev_read[dst], 0);
     if (e != cudaSuccess) return e;
-    e = launch_march(h->storage, march_args(h, src), &h->pmap[src], h->stream);
+    if (h->pass_kind == PASS_MARCH) {
+        e = launch_march(h->storage, march_args(h, src), &h->pmap[src], h->stream);
+        h->launches += 1;
+    } else {
+        const void *state[GROUP_STEPS + 1];
+        long long plane[GROUP_STEPS + 1];
+        pass_states(h, src, state, plane);
+        for (int j = 0; j < GROUP_STEPS && e == cudaSuccess; ++j) {
+            StepArgs a = step_args(h, src, dst, 0);
+            a.src = state[j];
+            a.dst = const_cast<void *>(state[j + 1]);
+            a.partials = pass_partials(h, src, j);
+            a.step_ctr = h->front + src;
+            a.step_off = j;
+            a.next_ctr = j == 0 ? h->front + dst : nullptr;
+            e = launch_collide_stream(h->storage, a, h->tiles_x, h->tiles_y, false, nullptr, h->stream);
+            h->launches += 1;
+        }
+    }
     h->lead_src = src;
     h->lead_pre = 0;
     h->lead_steps = GROUP_STEPS;
-    h->launches += 1;
     return e;
 }
 
@@ -540,15 +573,17 @@ lbm_status ensure_series(lbm_ctx *h, long long need)
     return LBM_OK;
 }
 
-// Decides whether the grid takes multi-step passes and lays out the rectangles
-// they treat apart, from the solid nodes' bounding box:
+// Decides how the grid takes passes and lays out the rectangles that the
+// multi-step kernel treats apart, from the solid nodes' bounding box:
 //   bounce: one node wider, which holds every node with a solid neighbour;
 //   keep:   where the link kernel and the control-volume sums read states:
 //           one node wider than that and than the box (pulled neighbours).
 // A rectangle that touches the top or bottom edge covers all rows (y wraps).
 void plan_passes(lbm_ctx *h, const std::vector<long long> &solids)
 {
-    h->march = false;
+    const int all[4] = {0, h->nx - 1, 0, h->ny - 1};
+    memcpy(h->keep, all, sizeof(all));  // single steps keep whole states
+    h->pass_kind = 9.0 * (double)h->plane * (double)h->elem <= PASS_STATE_BYTES ? PASS_STEPS : PASS_NONE;
     if (h->periodic || !march_grid(h->storage, h->nx, h->ny)) return;
     int x0 = h->nx, x1 = -1, y0 = h->ny, y1 = -1;
     for (long long n : solids) {
@@ -579,29 +614,34 @@ void plan_passes(lbm_ctx *h, const std::vector<long long> &solids)
         k[2] = 0;
         k[3] = h->ny - 1;
     }
-    memcpy(h->keep, k, sizeof(k));
     if ((double)(k[1] - k[0] + 1) * (k[3] - k[2] + 1) > MARCH_KEEP_SHARE * h->nx * h->ny) return;
-    h->march = true;
+    memcpy(h->keep, k, sizeof(k));
+    h->pass_kind = PASS_MARCH;
 }
 
-// The buffers of the multi-step passes, at first use.  Without room for them
+// The buffers of the passes, at first use.  Without room for them
 // the handle takes single steps.
 void ensure_passes(lbm_ctx *h)
 {
-    if (!h->march || h->mid) return;
+    if (h->pass_kind == PASS_NONE || h->mid) return;
     const size_t state = 9 * (size_t)mid_plane(h) * h->elem;
     h->mid = (char *)dev_alloc(h, state * NBUF * (GROUP_STEPS - 1));
-    h->group_partials = (double *)dev_alloc(h, sizeof(double) * GROUP_STEPS * CV_PARTIAL * h->n_cv_tiles);
-    std::vector<int2> units;
-    h->plan = march_plan(h->storage, h->nx, h->ny, h->sm_count, h->bounce, h->keep, &units);
-    h->n_units = (int)units.size();
-    h->march_units_d = (int2 *)dev_alloc(h, sizeof(int2) * units.size());
-    bool ok = h->mid && h->group_partials && h->march_units_d;
-    ok = ok && cudaMemcpyAsync(h->march_units_d, units.data(), sizeof(int2) * units.size(), cudaMemcpyHostToDevice,
-                               h->stream) == cudaSuccess &&
-         cudaStreamSynchronize(h->stream) == cudaSuccess;
-    for (int b = 0; b < NBUF; ++b)
-        ok = ok && encode_tensor_map(&h->pmap[b], h->storage, h->pop[b], h->pitch, h->ny, march_box_columns(h->storage), 1);
+    h->group_partials = (double *)dev_alloc(h, sizeof(double) * NBUF * GROUP_STEPS * CV_PARTIAL * h->n_cv_tiles);
+    // the kernels' copies and prefetches of rows start on 16-byte boundaries
+    bool ok = h->mid && h->group_partials && ((uintptr_t)h->mid & 15) == 0;
+    if (ok && h->pass_kind == PASS_MARCH) {
+        std::vector<int2> units;
+        h->plan = march_plan(h->storage, h->nx, h->ny, h->sm_count, h->bounce, h->keep, &units);
+        h->n_units = (int)units.size();
+        h->march_units_d = (int2 *)dev_alloc(h, sizeof(int2) * units.size());
+        ok = h->march_units_d &&
+             cudaMemcpyAsync(h->march_units_d, units.data(), sizeof(int2) * units.size(), cudaMemcpyHostToDevice,
+                             h->stream) == cudaSuccess &&
+             cudaStreamSynchronize(h->stream) == cudaSuccess;
+        for (int b = 0; b < NBUF; ++b)
+            ok = ok && encode_tensor_map(&h->pmap[b], h->storage, h->pop[b], h->pitch, h->ny,
+                                         march_box_columns(h->storage), 1);
+    }
     if (!ok) {
         dev_free(h, h->mid);
         dev_free(h, h->group_partials);
@@ -609,7 +649,7 @@ void ensure_passes(lbm_ctx *h)
         h->mid = nullptr;
         h->group_partials = nullptr;
         h->march_units_d = nullptr;
-        h->march = false;
+        h->pass_kind = PASS_NONE;
     }
 }
 
@@ -836,7 +876,7 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
     h->link_totals = h->link_partials + link_rows;
     ALLOC(h->ticket, unsigned int *, sizeof(unsigned int) * 16);
     ALLOC(h->carry, double *, sizeof(double) * 8);
-    ALLOC(h->step_ctr, long long *, sizeof(long long) * 2);
+    ALLOC(h->step_ctr, long long *, sizeof(long long) * (1 + NBUF));
     h->front = h->step_ctr + 1;
     ALLOC(h->status, int *, sizeof(int) * 2);
     st = ensure_series(h, 1024);
@@ -851,7 +891,7 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
     CKC(cudaMemsetAsync(h->partials, 0, sizeof(double) * NBUF * CV_PARTIAL * h->n_cv_tiles, s), "memset");
     CKC(cudaMemsetAsync(h->ticket, 0, sizeof(unsigned int) * 16, s), "memset");
     CKC(cudaMemsetAsync(h->carry, 0, sizeof(double) * 8, s), "memset");
-    CKC(cudaMemsetAsync(h->step_ctr, 0, sizeof(long long) * 2, s), "memset");
+    CKC(cudaMemsetAsync(h->step_ctr, 0, sizeof(long long) * (1 + NBUF), s), "memset");
     const int status0[2] = {0, INT_MAX};
     CKC(cudaMemcpyAsync(h->status, status0, sizeof(status0), cudaMemcpyHostToDevice, s), "H2D status");
     h->status_armed = true;
@@ -967,14 +1007,14 @@ lbm_status queue_steps(lbm_ctx *h, int n)
     int nev = 0;
     if (n >= GROUP_STEPS) ensure_passes(h);
     while (n > 0) {
-        const bool marching = h->march && !h->use_bulk && !h->timing;
-        const bool pass = marching && !h->precollision && n >= GROUP_STEPS;
+        const bool passes = h->pass_kind != PASS_NONE && !h->use_bulk && !h->timing;
+        const bool pass = passes && !h->precollision && n >= GROUP_STEPS;
         if (pass && h->front_host != h->t) {
-            CK(h, launch_set_front(h->front, h->t, h->stream), "step counter");
+            CK(h, launch_set_counter(h->front + h->cur, h->t, h->stream), "step counter");
             h->front_host = h->t;
             h->launches += 1;
         }
-        if (pass ? n < NBUF * GROUP_STEPS : (h->precollision || h->timing || n < NBUF || marching)) {
+        if (pass ? n < NBUF * GROUP_STEPS : (h->precollision || h->timing || n < NBUF || passes)) {
             cudaEvent_t *ev = h->timing ? &h->events[3 * nev] : nullptr;
             CK(h, pass ? launch_one_pass(h, h->cur) : launch_one_step(h, h->cur, h->precollision, ev), "step launch");
             if (h->timing && ++nev == TIMING_BATCH) {
@@ -1005,7 +1045,10 @@ lbm_status queue_steps(lbm_ctx *h, int n)
             h->lead_src = prev_buf(h->cur);  // units is a multiple of NBUF
             h->lead_pre = 0;
             h->lead_steps = each;
-            h->launches += (pass ? 3 : 2) * (long long)units - (pass ? 2 : 1) * (1 - lead);  // the last link kernel is held
+            // the last link kernel (after a multi-step pass, the box sums, too) is held
+            const int own = !pass || h->pass_kind == PASS_MARCH ? 1 : GROUP_STEPS;
+            const int link = pass && h->pass_kind == PASS_MARCH ? 2 : 1;
+            h->launches += (long long)(own + link) * units - link * (1 - lead);
             h->t += (long long)units * each;
             if (pass) h->front_host += (long long)units * each;
             n -= units * each;
@@ -1187,7 +1230,7 @@ lbm_status lbm_prepare(lbm_ctx *h, long n)
     lbm_status st = ensure_series(h, h->t + n);
     if (st != LBM_OK) return st;
     ensure_passes(h);
-    const bool pass = h->march && !h->use_bulk;  // such a handle replays no graph of single steps
+    const bool pass = h->pass_kind != PASS_NONE && !h->use_bulk;  // such a handle replays no graph of single steps
     for (int p = 0; p < NBUF; ++p)
         for (int k = 0; k < 2; ++k)
             for (int l = 0; l < 2; ++l)

@@ -154,6 +154,8 @@ struct StepArgs {
     int pf_rows;             // L2 prefetch distance of the direct kernel in tile rows (0: off)
     int first_r0, first_r1;  // tile rows with bounce-back tiles, dispatched first (r0 > r1: none)
     unsigned int wait_limit; // polls of each pipeline wait of the staged kernel (WAIT_LIMIT)
+    int step_off;            // this launch's step is *step_ctr + step_off
+    long long *next_ctr;     // receives *step_ctr + GROUP_STEPS (NULL: nothing): the counter of the next pass
 };
 
 // The relaxation rate of a StepArgs: the FP64 value and its FP32 rounding (a

@@ -12,7 +12,7 @@ constexpr int MARCH_STEPS = GROUP_STEPS;  // steps of one pass
 constexpr int MARCH_HALO = 4;             // columns computed but not stored on each side of a strip (>= steps - 1)
 
 struct MarchArgs {
-    StepArgs s;                  // src = b(t), dst = b(t + steps); grid, boundary and collision parameters
+    StepArgs s;                  // src = b(t), dst = b(t + steps); grid, boundary and collision parameters; the counters
     void *mid[MARCH_STEPS - 1];  // b(t + 1) .. b(t + steps - 1), rows keep[2]..keep[3] of the grid
     long long mid_plane;         // elements between two planes of a mid buffer
     int out_w;                   // columns a strip stores
@@ -20,8 +20,6 @@ struct MarchArgs {
     int n_units;
     int bounce[4];               // columns x0..x1, rows y0..y1 with a solid node in them or next to them (x0 > x1: none)
     int keep[4];                 // columns x0..x1, rows y0..y1 whose intermediate states are stored (x0 > x1: none)
-    long long *front;            // steps done by the collide-stream kernels
-    unsigned int *ticket;        // arrival counter of the CTAs
 };
 
 // Strips of the multi-step kernel for a grid (each stores out_w columns) and
@@ -40,8 +38,8 @@ MarchPlan march_plan(int storage, int nx, int ny, int sm_count, const int *bounc
 // is march_box_columns(storage) columns of one row of all nine planes
 cudaError_t launch_march(int storage, const MarchArgs &a, const void *map, cudaStream_t st);
 int march_box_columns(int storage);
-// *front = t
-cudaError_t launch_set_front(long long *front, long long t, cudaStream_t st);
+// *ctr = t
+cudaError_t launch_set_counter(long long *ctr, long long t, cudaStream_t st);
 
 // Control-volume partial rows of the steps of a pass, as the single-step
 // kernel would have written them: step j reads state[j] and state[j + 1].

@@ -104,7 +104,11 @@ __global__ void __launch_bounds__((TILE_X / cols_per_thread(S)) * (tile_rows(S) 
                                   DirectMinBlocks<S>::value)
     k_collide_stream(StepArgs a)
 {
-    if constexpr (!MOMENTUM_ONLY) prefetch_ahead<S>(a);
+    if constexpr (!MOMENTUM_ONLY) {
+        prefetch_ahead<S>(a);
+        if (a.next_ctr && (blockIdx.x | blockIdx.y | threadIdx.x | threadIdx.y) == 0)
+            *a.next_ctr = *a.step_ctr + GROUP_STEPS;
+    }
     // a launch over a sub-rectangle of tiles (the momentum-only pass) keeps plain order
     const int tx = blockIdx.x + a.tile_off_x;
     const int ty = (MOMENTUM_ONLY || a.tile_off_y != 0) ? (int)blockIdx.y + a.tile_off_y
@@ -296,7 +300,7 @@ __global__ void __launch_bounds__(TmaCfg<S>::THREADS, GBLBM_TMA_MINB)
         const int any_bad = __syncthreads_or(bad);  // also: every read of stage s is done
         if (any_bad && threadIdx.x == 0) {
             atomicOr(a.status, 1);
-            atomicMin(a.status + 1, (int)*a.step_ctr);
+            atomicMin(a.status + 1, (int)*a.step_ctr + a.step_off);
         }
         if (threadIdx.x == 0 && k + C::NS < count) {
             tma::fence_proxy_async();
