@@ -27,7 +27,7 @@ struct AdjArgs {
     const void *lam_next;  // [9][ny][pitch] compute type: lam(t+1)
     void *lam;             // [9][ny][pitch] compute type: lam(t)
     const uint16_t *nbits;
-    const uint8_t *tile_flag;  // per tile of the grid: 0 = every node's bits are 0 (or NULL)
+    const uint8_t *tile_flag;  // per collide-stream tile: 0 = every node's bits are 0 (or NULL)
     const double *u_row;
     double *du_acc;        // [ny] running dJ/du_in
     double *dw_acc;        // [blocks * ADJ_WARPS] running per-warp dJ/domega: FP64, or a
@@ -213,14 +213,22 @@ __global__ void __launch_bounds__(ADJ_THREADS, GBLBM_ADJ_MINB) k_adjoint_step(Ad
 {
     using T = typename Traits<S>::comp_t;
     using Acc = typename AccOf<S>::type;
+    constexpr int ADJ_FLAGS = ADJ_TR / tile_rows(S);  // collide-stream tiles in a tile of this kernel
+    static_assert(ADJ_TR % tile_rows(S) == 0, "whole collide-stream tiles");
     T *__restrict__ lam = (T *)a.lam;
     adj_prefetch<S>(a);
     const int x = blockIdx.x * ADJ_TX + threadIdx.x;
     const int y0 = blockIdx.y * ADJ_TR + threadIdx.y * ADJ_RPT;
     // a tile whose nodes all have zero bits (no solid in or next to it) skips
     // the per-node bit loads, so its population loads start at once
-    const bool plain_tile =
-        a.tile_flag && !a.precollision && a.tile_flag[(long long)blockIdx.y * gridDim.x + blockIdx.x] == 0;
+    bool plain_tile = a.tile_flag && !a.precollision;
+    if (plain_tile) {
+#pragma unroll
+        for (int k = 0; k < ADJ_FLAGS; ++k) {
+            const int ty = (int)blockIdx.y * ADJ_FLAGS + k;
+            if (ty * (ADJ_TR / ADJ_FLAGS) < a.ny && a.tile_flag[(long long)ty * gridDim.x + blockIdx.x]) plain_tile = false;
+        }
+    }
     Acc dw;
     acc_zero(dw);
     if (x < a.nx) {
@@ -329,9 +337,10 @@ cudaError_t launch_adjoint_step(int storage, const void *src, int precollision, 
     }
     dim3 grid((nx + ADJ_TX - 1) / ADJ_TX, (ny + ADJ_TR - 1) / ADJ_TR);
     dim3 block(ADJ_TX, ADJ_TR / ADJ_RPT);
-    // the collide-stream tile flags serve when their tiles are these tiles
-    a.tile_flag = (tile_flag && TILE_X == ADJ_TX && flag_rows == ADJ_TR && flag_tiles_x == (int)grid.x) ? tile_flag
-                                                                                                        : nullptr;
+    // the collide-stream tile flags serve when whole ones make up these tiles
+    a.tile_flag = (tile_flag && TILE_X == ADJ_TX && flag_rows == tile_rows(storage) && flag_tiles_x == (int)grid.x)
+                      ? tile_flag
+                      : nullptr;
     // prefetch half the CTAs the GPU holds at once ahead, in tile rows
     int pf_rows = 0;
     if (storage != LBM_F64) {

@@ -56,7 +56,10 @@ constexpr double MARCH_KEEP_SHARE = 0.25;
 // with two link kernels in flight).  The second kind holds nine more states,
 // so it is for states of at most PASS_STATE_BYTES.
 enum PassKind { PASS_NONE = 0, PASS_MARCH, PASS_STEPS };
-constexpr double PASS_STATE_BYTES = 64e6;
+constexpr double PASS_STATE_BYTES = 14e6;
+// Steps of a pass follow one another early (StepArgs::early) up to this many
+// CTAs an SM.
+constexpr int EARLY_CTAS = 4;
 
 }  // namespace
 
@@ -484,6 +487,7 @@ cudaError_t launch_one_pass(lbm_ctx *h, int src)
             a.step_ctr = h->front + src;
             a.step_off = j;
             a.next_ctr = j == 0 ? h->front + dst : nullptr;
+            a.early = j > 0 && h->tiles_x * h->tiles_y <= EARLY_CTAS * h->sm_count;
             e = launch_collide_stream(h->storage, a, h->tiles_x, h->tiles_y, false, nullptr, h->stream);
             h->launches += 1;
         }

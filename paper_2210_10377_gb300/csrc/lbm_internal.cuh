@@ -59,9 +59,17 @@ constexpr int GROUP_STEPS = 4;
 #ifndef GBLBM_TR_F32
 #define GBLBM_TR_F32 4
 #endif
+// FP64: one row (128 threads).  Its tiles are bound by the SM's FP64 units (two
+// operations a clock), so a grid of a few thousand nodes has to reach all SMs:
+// 256 x 128 in tiles of 4 rows kept 64 of 152 busy.
+#ifndef GBLBM_TR_F64
+#define GBLBM_TR_F64 1
+#endif
 __host__ __device__ constexpr int tile_rows(int storage)
 {
-    return (storage == LBM_F32 || storage == LBM_F32_DEV) ? GBLBM_TR_F32 : (storage == LBM_F16_DEV ? GBLBM_TR_F16 : 4);
+    return (storage == LBM_F32 || storage == LBM_F32_DEV)
+               ? GBLBM_TR_F32
+               : (storage == LBM_F16_DEV ? GBLBM_TR_F16 : GBLBM_TR_F64);
 }
 // Adjacent columns per thread of the direct-load kernels: FP16 deviations
 // take two, so that loads and stores move 4-byte pairs (a tuning knob).
@@ -155,6 +163,7 @@ struct StepArgs {
     int first_r0, first_r1;  // tile rows with bounce-back tiles, dispatched first (r0 > r1: none)
     unsigned int wait_limit; // polls of each pipeline wait of the staged kernel (WAIT_LIMIT)
     int step_off;            // this launch's step is *step_ctr + step_off
+    int early;               // launched while its predecessor may still run (see launch_collide_stream)
     long long *next_ctr;     // receives *step_ctr + GROUP_STEPS (NULL: nothing): the counter of the next pass
 };
 

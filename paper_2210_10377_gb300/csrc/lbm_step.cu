@@ -104,17 +104,21 @@ __global__ void __launch_bounds__((TILE_X / cols_per_thread(S)) * (tile_rows(S) 
                                   DirectMinBlocks<S>::value)
     k_collide_stream(StepArgs a)
 {
-    if constexpr (!MOMENTUM_ONLY) {
-        prefetch_ahead<S>(a);
-        if (a.next_ctr && (blockIdx.x | blockIdx.y | threadIdx.x | threadIdx.y) == 0)
-            *a.next_ctr = *a.step_ctr + GROUP_STEPS;
-    }
-    // a launch over a sub-rectangle of tiles (the momentum-only pass) keeps plain order
+    // the next step's CTAs may be placed; they wait here for this grid's end
+    // before they read or write anything this one does
+    if constexpr (!MOMENTUM_ONLY) asm volatile("griddepcontrol.launch_dependents;");
     const int tx = blockIdx.x + a.tile_off_x;
     const int ty = (MOMENTUM_ONLY || a.tile_off_y != 0) ? (int)blockIdx.y + a.tile_off_y
                                                         : tile_row_of((int)blockIdx.y, (int)gridDim.y,
                                                                       a.first_r0, a.first_r1);
+    // a launch over a sub-rectangle of tiles (the momentum-only pass) keeps plain order
     const bool checked = a.precollision || a.tile_flag[(long long)ty * a.tiles_x + tx] != 0;
+    if constexpr (!MOMENTUM_ONLY) {
+        if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+        prefetch_ahead<S>(a);
+        if (a.next_ctr && (blockIdx.x | blockIdx.y | threadIdx.x | threadIdx.y) == 0)
+            *a.next_ctr = *a.step_ctr + GROUP_STEPS;
+    }
     collide_tile<S, MOMENTUM_ONLY, FORCE, TILE_X, tile_rows(S), direct_rpt(S)>(a, tx, ty, checked);
 }
 
@@ -386,21 +390,31 @@ cudaError_t launch_collide_stream(int storage, const StepArgs &a, int tiles_x, i
     dim3 grid(tiles_x, tiles_y);
     const bool force = a.gx != 0.0 || a.gy != 0.0;
     dim3 block(TILE_X / cols_per_thread(storage), tile_rows(storage) / direct_rpt(storage));
-#define GBLBM_CS(S)                                                    \
-    if (momentum_only)                                                 \
-        k_collide_stream<S, true, false><<<grid, block, 0, st>>>(a);   \
-    else if (force)                                                    \
-        k_collide_stream<S, false, true><<<grid, block, 0, st>>>(a);   \
-    else                                                               \
-        k_collide_stream<S, false, false><<<grid, block, 0, st>>>(a);
+    // An early launch (a.early) is a programmatic dependent of the launch
+    // before it on the stream: its CTAs are placed while that one drains, and
+    // wait for its end where they start to touch populations.  That hides the
+    // launch latency between the steps of a small grid; on a grid that fills
+    // the GPU the waiting CTAs would keep the link kernel's out.
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = a.early ? 1 : 0;
+#define GBLBM_CS(S)                                                                                       \
+    return momentum_only ? cudaLaunchKernelEx(&cfg, k_collide_stream<S, true, false>, a)                  \
+           : force       ? cudaLaunchKernelEx(&cfg, k_collide_stream<S, false, true>, a)                  \
+                         : cudaLaunchKernelEx(&cfg, k_collide_stream<S, false, false>, a)
     switch (storage) {
-    case LBM_F64: GBLBM_CS(LBM_F64); break;
-    case LBM_F32: GBLBM_CS(LBM_F32); break;
-    case LBM_F32_DEV: GBLBM_CS(LBM_F32_DEV); break;
-    default: GBLBM_CS(LBM_F16_DEV); break;
+    case LBM_F64: GBLBM_CS(LBM_F64);
+    case LBM_F32: GBLBM_CS(LBM_F32);
+    case LBM_F32_DEV: GBLBM_CS(LBM_F32_DEV);
+    default: GBLBM_CS(LBM_F16_DEV);
     }
 #undef GBLBM_CS
-    return cudaGetLastError();
 }
 
 }  // namespace gblbm
