@@ -60,6 +60,8 @@ constexpr double PASS_STATE_BYTES = 14e6;
 // Steps of a pass follow one another early (StepArgs::early) up to this many
 // CTAs an SM.
 constexpr int EARLY_CTAS = 4;
+// States up to this size are read back through one scratch array and copy.
+constexpr size_t READ_TOGETHER_BYTES = (size_t)32 << 20;
 
 }  // namespace
 
@@ -1295,22 +1297,33 @@ lbm_status lbm_populations(lbm_ctx *h, double *out)
     SETTLE(h);
     if (!out) return set_err(h, LBM_EINVAL, "out must not be NULL");
     const size_t N = (size_t)h->nx * h->ny;
-    double *scratch = (double *)dev_alloc(h, sizeof(double) * N);
+    // Two scratch planes: while one plane is copied to the host on the side
+    // stream, the next one is gathered on the handle's.  Small planes are
+    // gathered together and copied at once.
+    const bool together = 9 * sizeof(double) * N <= READ_TOGETHER_BYTES;
+    double *scratch = (double *)dev_alloc(h, sizeof(double) * N * (together ? 9 : 2));
     if (!scratch) return set_err(h, LBM_ENOMEM, "scratch allocation failed");
-    lbm_status st = LBM_OK;
-    for (int i = 0; i < 9 && st == LBM_OK; ++i) {
-        cudaError_t e = launch_gather(h->storage, h->pop[h->cur], h->nbits, h->inlet, h->plane, h->nx,
-                                      h->ny, h->pitch, h->periodic, h->precollision, h->rho0, i,
-                                      scratch, h->stream);
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 9 && e == cudaSuccess; ++i) {
+        double *plane = scratch + (together ? i : i & 1) * N;
+        if (!together && i >= 2) e = cudaStreamWaitEvent(h->stream, h->ev_read[i & 1], 0);
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(out + i * N, scratch, sizeof(double) * N, cudaMemcpyDeviceToHost,
-                                h->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-        if (e != cudaSuccess) st = cuda_err(h, e, "gather populations");
+            e = launch_gather(h->storage, h->pop[h->cur], h->nbits, h->inlet, h->plane, h->nx, h->ny, h->pitch,
+                              h->periodic, h->precollision, h->rho0, i, plane, h->stream);
         h->launches += 1;
+        if (together) continue;
+        if (e == cudaSuccess) e = cudaEventRecord(h->ev_fork, h->stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->ev_fork, 0);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(out + i * N, plane, sizeof(double) * N, cudaMemcpyDeviceToHost, h->side);
+        if (e == cudaSuccess) e = cudaEventRecord(h->ev_read[i & 1], h->side);
     }
+    if (e == cudaSuccess && together)
+        e = cudaMemcpyAsync(out, scratch, sizeof(double) * 9 * N, cudaMemcpyDeviceToHost, h->stream);
+    const cudaError_t e1 = cudaStreamSynchronize(h->side), e2 = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess) e = e1 != cudaSuccess ? e1 : e2;
     dev_free(h, scratch);
-    return st;
+    return e == cudaSuccess ? LBM_OK : cuda_err(h, e, "gather populations");
 }
 
 lbm_status lbm_set_populations(lbm_ctx *h, const double *in)
