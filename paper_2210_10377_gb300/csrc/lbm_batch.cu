@@ -81,7 +81,7 @@ __device__ __forceinline__ void batch_tile(const BatchParams &p, int k)
         }
         a.use_bulk = 0;
         a.sm_count = 0;
-        a.step_off = 0;
+        a.step_off = p.step_off;
         a.early = 0;
         a.next_ctr = nullptr;
         collide_tile<S, MOMENTUM_ONLY, false, TX, TR, RPT>(a, e.y, e.z, p.precollision || e.w != 0);
@@ -94,6 +94,8 @@ template <int S, bool MOMENTUM_ONLY, bool PERSIST, int TX, int TR, int RPT>
 __global__ void __launch_bounds__((TX / cols_per_thread(S)) * (TR / RPT), PERSIST ? 0 : BatchMinBlocks<S>::value)
     k_collide_stream_batch(const __grid_constant__ BatchParams p)
 {
+    if (!MOMENTUM_ONLY && p.next_ctr && (blockIdx.x | threadIdx.x | threadIdx.y) == 0)
+        *p.next_ctr = *p.step_ctr + GROUP_STEPS;
     if (PERSIST) {
         for (int k = blockIdx.x; k < p.n_tiles; k += gridDim.x) batch_tile<S, MOMENTUM_ONLY, TX, TR, RPT>(p, k);
     } else if ((int)blockIdx.x < p.n_tiles) {

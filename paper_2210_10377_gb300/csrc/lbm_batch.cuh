@@ -88,6 +88,8 @@ struct BatchParams {
     int periodic;
     int precollision;        // the state is pre-collision (first step)
     int cv_only;             // momentum-only pass over the control-volume tiles
+    int step_off;            // this launch's step is *step_ctr + step_off
+    long long *next_ctr;     // receives *step_ctr + GROUP_STEPS (NULL: nothing)
     double rho0;
     float rho0_f;
     BatchDomain dom[MAX_BATCH_DOMAINS];
@@ -95,7 +97,10 @@ struct BatchParams {
 static_assert(sizeof(BatchParams) <= 32000, "kernel parameter block above the 32 KB limit");
 
 struct BatchLinkArgs {
-    const LinkArgs *args;     // [n_domains]: this step's link arguments of every domain
+    const LinkArgs *args;     // [steps][n_domains]: the link arguments of every domain and step
+    int steps;                // consecutive steps of this launch
+    double *totals;           // [n_domains][GROUP_STEPS][16]: the reduced sums (steps > 1)
+    unsigned int *tickets;    // [n_domains]: arrival counters of a domain's steps (steps > 1)
     double *series;           // [rows][n_domains][SERIES_ROW]
     long long series_rows;
     int n_domains;
@@ -112,6 +117,7 @@ cudaError_t launch_collide_stream_batch(int storage, int shape, bool momentum_on
                                         const BatchParams &p, int grid, cudaStream_t st);
 // Resident CTAs per SM of the persistent batched kernel for (storage, shape), or 0.
 int batch_max_ctas_per_sm(int storage, int shape);
-cudaError_t launch_link_force_batch(int storage, const BatchLinkArgs &b, cudaStream_t st);
+// priority: as launch_link_force
+cudaError_t launch_link_force_batch(int storage, const BatchLinkArgs &b, cudaStream_t st, int priority = 0);
 
 }  // namespace gblbm

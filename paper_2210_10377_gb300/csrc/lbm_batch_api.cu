@@ -4,9 +4,11 @@
 // tuner and read-back.  All arithmetic of the method runs in the kernels of
 // lbm_setup.cu, lbm_batch.cu and lbm_link.cu.
 //
-// Two population buffers alternate: step t reads buffer t % 2 and writes the
-// other; the link kernel of step t runs after the collide-stream kernel on the
-// same stream, so the buffer of step t-1 is free again once step t is done.
+// Two population buffers alternate: a single step reads one and writes the
+// other; its link kernel runs after the collide-stream kernel on the same
+// stream.  Batches whose arenas are small enough take GROUP_STEPS steps a
+// pass: the steps in between write arenas of their own, and one link kernel
+// for all of them runs beside the next pass on a side stream.
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -20,6 +22,7 @@
 #include "lbm_batch.cuh"
 #include "lbm_host.h"
 #include "lbm_internal.cuh"
+#include "lbm_march.cuh"
 
 using namespace gblbm;
 
@@ -38,6 +41,14 @@ namespace {
 #define GBLBM_BATCH_PATH_ORDER_F32 0
 #endif
 constexpr int BATCH_GRAPH_STEPS = 16;  // steps per captured graph (even: ends on the start buffer)
+// Passes per captured graph (even: ends on the start buffer).
+constexpr int BATCH_GRAPH_PASSES[2] = {8, 2};
+// Batches up to this arena size take passes (six arenas more).  A link kernel
+// after every step, alone on the GPU for its 15-20 us, was half the step of
+// the cylinder study's batch (35 MB: 25 us a step) and a third of 12 airfoil
+// domains' (62 us), but 2 % of 256 domains' (2.4 GB).
+constexpr size_t BATCH_PASS_BYTES = (size_t)192 << 20;
+constexpr size_t BATCH_GUARD_FRONT = 256;  // bytes before an arena's first element
 constexpr int BATCH_GRID_CHOICES[] = {1, 2, 3, 4, 6, 8};  // persistent CTAs per SM tried by the tuner
 
 struct Domain {
@@ -104,6 +115,24 @@ struct lbm_batch {
     int cur = 0;
     int shape = 0, ctas_per_sm = 0;
     cudaGraphExec_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
+    // passes (allocated at first use; pass_ok: the batch takes them)
+    bool pass_ok = false;
+    size_t arena_bytes = 0;       // one population arena with its guards
+    long long part_rows = 0;      // rows of one partials slice
+    char *mid = nullptr;          // [2][GROUP_STEPS - 1] arenas: the steps in between of the pass from each buffer
+    double *pass_partials = nullptr;  // [2][GROUP_STEPS] slices
+    LinkArgs *pass_largs = nullptr;   // [BATCH_SHAPES][2][GROUP_STEPS][n]
+    double *totals = nullptr;         // [n][GROUP_STEPS][16]
+    unsigned int *tickets = nullptr;  // [n]
+    long long *front = nullptr;       // [2] the step at which the pass from each buffer starts
+    long long front_host = -1;
+    cudaStream_t side = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_read = nullptr;
+    bool read_live = false;       // a link kernel of a pass is on the side stream
+    int held = -1;                // the pass whose link kernel is not queued yet (its source buffer)
+    int link_prio = 0;
+    // [start buffer][BATCH_GRAPH_PASSES][opens with the previous pass's link kernel]
+    cudaGraphExec_t pass_graph[2][2][2] = {};
     long long launches = 0;
     std::string err;
 };
@@ -167,6 +196,13 @@ void drop_graphs(lbm_batch *b)
                 cudaGraphExecDestroy(b->graph[c][k]);
                 b->graph[c][k] = nullptr;
             }
+    for (int c = 0; c < 2; ++c)
+        for (int k = 0; k < 2; ++k)
+            for (int l = 0; l < 2; ++l)
+                if (b->pass_graph[c][k][l]) {
+                    cudaGraphExecDestroy(b->pass_graph[c][k][l]);
+                    b->pass_graph[c][k][l] = nullptr;
+                }
 }
 
 void free_all(lbm_batch *b)
@@ -177,8 +213,11 @@ void free_all(lbm_batch *b)
                     b->links, b->bnodes, b->partials, b->tune_partials, b->checked[0], b->checked[1],
                     b->checked[2], b->checked_cv[0], b->checked_cv[1], b->checked_cv[2], b->largs,
                     b->series, b->carry, b->step_ctr, b->ticket, b->status, b->tune_status,
-                    b->bstatus};
+                    b->bstatus, b->mid, b->pass_partials, b->pass_largs, b->totals, b->tickets, b->front};
     for (void *p : bufs) bdev_free(b, p);
+    for (cudaEvent_t e : {b->ev_fork, b->ev_join, b->ev_read})
+        if (e) cudaEventDestroy(e);
+    if (b->side) cudaStreamDestroy(b->side);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
 }
 
@@ -268,6 +307,18 @@ LinkArgs link_args(const lbm_batch *b, int d, int s, int src)
     return a;
 }
 
+// Population arena of step j of the pass from buffer c (0: its source,
+// GROUP_STEPS: its result), and the partials slice of its step j.
+char *pass_state(const lbm_batch *b, int c, int j)
+{
+    if (j == 0 || j == GROUP_STEPS) return b->pop[j == 0 ? c : 1 - c];
+    return b->mid + ((size_t)c * (GROUP_STEPS - 1) + (j - 1)) * b->arena_bytes + BATCH_GUARD_FRONT;
+}
+double *pass_slice(const lbm_batch *b, int c, int j)
+{
+    return b->pass_partials + ((size_t)c * GROUP_STEPS + j) * CV_PARTIAL * b->part_rows;
+}
+
 // Table index of (shape, slot, domain); slot 0/1 = source buffer, 2 = first step.
 size_t tix(const lbm_batch *b, int s, int slot) { return ((size_t)s * 3 + slot) * b->n; }
 
@@ -305,18 +356,69 @@ lbm_status ensure_series(lbm_batch *b, long long need)
     return LBM_OK;
 }
 
+// The buffers of the passes, at first use.  Without room for them the batch
+// takes single steps.
+lbm_status ensure_passes(lbm_batch *b)
+{
+    if (!b->pass_ok || b->mid) return LBM_OK;
+    const size_t n = (size_t)b->n, slices = 2 * (size_t)GROUP_STEPS;
+    b->mid = (char *)bdev_alloc(b, 2 * (GROUP_STEPS - 1) * b->arena_bytes);
+    b->pass_partials = (double *)bdev_alloc(b, sizeof(double) * slices * CV_PARTIAL * b->part_rows);
+    b->pass_largs = (LinkArgs *)bdev_alloc(b, sizeof(LinkArgs) * BATCH_SHAPES * slices * n);
+    b->totals = (double *)bdev_alloc(b, sizeof(double) * n * GROUP_STEPS * 16);
+    b->tickets = (unsigned int *)bdev_alloc(b, sizeof(unsigned int) * n);
+    b->front = (long long *)bdev_alloc(b, sizeof(long long) * 2);
+    int least = 0;
+    cudaError_t e = cudaDeviceGetStreamPriorityRange(&least, &b->link_prio);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->side, cudaStreamNonBlocking, b->link_prio);
+    for (cudaEvent_t *ev : {&b->ev_fork, &b->ev_join, &b->ev_read})
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+    if (e != cudaSuccess || !b->mid || ((uintptr_t)b->mid & 15) || !b->pass_partials || !b->pass_largs || !b->totals ||
+        !b->tickets || !b->front) {
+        cudaGetLastError();
+        b->pass_ok = false;  // what was handed out is given back with the batch
+        return LBM_OK;
+    }
+    std::vector<LinkArgs> la(BATCH_SHAPES * slices * n);
+    for (int s = 0; s < BATCH_SHAPES; ++s)
+        for (int c = 0; c < 2; ++c)
+            for (int j = 0; j < GROUP_STEPS; ++j)
+                for (int d = 0; d < b->n; ++d) {
+                    LinkArgs a = link_args(b, d, s, c);
+                    const long long off = b->dom[d].pop_off * (long long)b->elem;
+                    a.src = pass_state(b, c, j) + off;
+                    a.dst = pass_state(b, c, j + 1) + off;
+                    a.partials = pass_slice(b, c, j) + CV_PARTIAL * b->dom[d].cvp_off[s];
+                    la[(((size_t)s * 2 + c) * GROUP_STEPS + j) * n + d] = a;
+                }
+    BCK(b, cudaMemcpyAsync(b->pass_largs, la.data(), sizeof(LinkArgs) * la.size(), cudaMemcpyHostToDevice, b->stream),
+        "H2D link tables");
+    BCK(b, cudaMemsetAsync(b->tickets, 0, sizeof(unsigned int) * n, b->stream), "memset");
+    BCK(b, cudaStreamSynchronize(b->stream), "sync");
+    return LBM_OK;
+}
+
 // Grid of the collide-stream launch: 0 = one CTA per tile, else persistent.
 int grid_of(const lbm_batch *b) { return b->ctas_per_sm > 0 ? b->ctas_per_sm * b->sm_count : 0; }
 
 // The collide-stream launches (one per chunk of domains) of a step reading
-// buffer src, or of the momentum pass.
-cudaError_t launch_collide(lbm_batch *b, int src, bool cv_only, bool tune, int shape, int grid)
+// buffer src, of the momentum pass, or of step pass_step (>= 0) of the pass
+// from buffer src.
+cudaError_t launch_collide(lbm_batch *b, int src, bool cv_only, bool tune, int shape, int grid, int pass_step = -1)
 {
     BatchParams *p = new (std::nothrow) BatchParams;
     if (!p) return cudaErrorMemoryAllocation;
     cudaError_t e = cudaSuccess;
     for (int c = 0; c < n_chunks(b) && e == cudaSuccess; ++c) {
         make_params(b, shape, src, c, cv_only, tune, *p);
+        if (pass_step >= 0) {
+            p->src = pass_state(b, src, pass_step);
+            p->dst = pass_state(b, src, pass_step + 1);
+            p->partials = pass_slice(b, src, pass_step);
+            p->step_ctr = b->front + src;
+            p->step_off = pass_step;
+            p->next_ctr = pass_step == 0 && c == 0 ? b->front + (1 - src) : nullptr;
+        }
         e = launch_collide_stream_batch(b->storage, shape, cv_only, *p, cv_only ? 0 : grid, b->stream);
         b->launches += 1;
     }
@@ -327,7 +429,9 @@ cudaError_t launch_collide(lbm_batch *b, int src, bool cv_only, bool tune, int s
 BatchLinkArgs link_launch_args(lbm_batch *b, int slot, bool drtt_only)
 {
     BatchLinkArgs bl;
+    memset(&bl, 0, sizeof(bl));
     bl.args = b->largs + tix(b, b->shape, slot);
+    bl.steps = 1;
     bl.series = b->series;
     bl.series_rows = b->series_cap;
     bl.n_domains = b->n;
@@ -349,26 +453,79 @@ cudaError_t launch_step(lbm_batch *b, int src)
     return e;
 }
 
-lbm_status build_graph(lbm_batch *b, int c, int k)
+// The held link kernel, if any, on the side stream after everything queued so
+// far on the batch's stream (its pass included).
+cudaError_t flush_link(lbm_batch *b)
 {
-    const int steps = k == 0 ? BATCH_GRAPH_STEPS : 2;
+    if (b->held < 0) return cudaSuccess;
+    const int c = b->held;
+    b->held = -1;
+    BatchLinkArgs bl = link_launch_args(b, 0, false);
+    bl.args = b->pass_largs + ((size_t)b->shape * 2 + c) * GROUP_STEPS * b->n;
+    bl.steps = GROUP_STEPS;
+    bl.totals = b->totals;
+    bl.tickets = b->tickets;
+    cudaError_t e = cudaEventRecord(b->ev_fork, b->stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side, b->ev_fork, 0);
+    if (e == cudaSuccess) e = launch_link_force_batch(b->storage, bl, b->side, b->link_prio);
+    if (e == cudaSuccess) e = cudaEventRecord(b->ev_read, b->side);
+    b->read_live = true;
+    b->launches += 1;
+    return e;
+}
+
+cudaError_t join_side(lbm_batch *b)
+{
+    if (!b->side) return cudaSuccess;
+    cudaError_t e = cudaEventRecord(b->ev_join, b->side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->ev_join, 0);
+    b->read_live = false;
+    return e;
+}
+
+// One pass from buffer c into the other one, its link kernel held.  The link
+// kernel of the pass before reads the buffer that the last step overwrites.
+cudaError_t launch_pass(lbm_batch *b, int c)
+{
+    cudaError_t e = flush_link(b);
+    for (int j = 0; j < GROUP_STEPS && e == cudaSuccess; ++j) {
+        if (j == GROUP_STEPS - 1 && b->read_live) e = cudaStreamWaitEvent(b->stream, b->ev_read, 0);
+        if (e == cudaSuccess) e = launch_collide(b, c, false, false, b->shape, grid_of(b), j);
+    }
+    b->held = c;
+    return e;
+}
+
+// Captures BATCH_GRAPH_STEPS (k = 0) or 2 steps, or BATCH_GRAPH_PASSES[k]
+// passes, from buffer c.  lead: the graph opens with the held link kernel of
+// the pass before.  A graph of passes ends with its last link kernel held.
+lbm_status build_graph(lbm_batch *b, int c, int k, bool passes, int lead)
+{
+    const int units = passes ? BATCH_GRAPH_PASSES[k] : (k == 0 ? BATCH_GRAPH_STEPS : 2);
     cudaGraph_t g = nullptr;
-    BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
     const long long saved = b->launches;
+    const int saved_held = b->held;
+    if (passes) b->held = lead ? 1 - c : -1;
+    b->read_live = false;
+    BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
     cudaError_t le = cudaSuccess;
     int src = c;
-    for (int s = 0; s < steps && le == cudaSuccess; ++s) {
-        le = launch_step(b, src);
+    for (int s = 0; s < units && le == cudaSuccess; ++s) {
+        le = passes ? launch_pass(b, src) : launch_step(b, src);
         src = 1 - src;
     }
+    if (le == cudaSuccess && passes && b->read_live) le = join_side(b);
+    b->read_live = false;
     b->launches = saved;
+    b->held = saved_held;
     cudaError_t ee = cudaStreamEndCapture(b->stream, &g);
     if (le != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
         return bcuda(b, le, "capture batch steps");
     }
     if (ee != cudaSuccess) return bcuda(b, ee, "end capture");
-    cudaError_t ie = cudaGraphInstantiate(&b->graph[c][k], g, 0);
+    cudaError_t ie = cudaGraphInstantiateWithFlags(passes ? &b->pass_graph[c][k][lead] : &b->graph[c][k], g,
+                                                   passes ? cudaGraphInstantiateFlagUseNodePriority : 0);
     cudaGraphDestroy(g);
     if (ie != cudaSuccess) return bcuda(b, ie, "instantiate graph");
     return LBM_OK;
@@ -513,8 +670,11 @@ lbm_status lbm_batch_create(const lbm_domain *domains, int n, const lbm_bc *bc_i
     long long cvp_max = 0;
     for (int s = 0; s < BATCH_SHAPES; ++s) cvp_max = cvp[s] > cvp_max ? cvp[s] : cvp_max;
 
-    const size_t guard_front = 256, guard_back = 2048;
+    const size_t guard_front = BATCH_GUARD_FRONT, guard_back = 2048;
     const size_t pop_bytes = (size_t)pop_elems * b->elem;
+    b->arena_bytes = (guard_front + pop_bytes + guard_back + 255) & ~(size_t)255;
+    b->part_rows = cvp_max > 0 ? cvp_max : 1;
+    b->pass_ok = b->arena_bytes <= BATCH_PASS_BYTES;
     for (int c = 0; c < 2; ++c) {
         BALLOC(b->pop_base[c], void *, guard_front + pop_bytes + guard_back);
         b->pop[c] = (char *)b->pop_base[c] + guard_front;
@@ -740,9 +900,44 @@ lbm_status lbm_batch_step(lbm_batch *b, int n)
     if (n == 0) return LBM_OK;
     lbm_status st = ensure_series(b, b->t + n);
     if (st != LBM_OK) return st;
+    if (n >= GROUP_STEPS) {
+        st = ensure_passes(b);
+        if (st != LBM_OK) return st;
+    }
     while (n > 0) {
-        if (b->t == 0 || n < 2) {
-            // the first step reads the pre-collision state; single steps run directly
+        const bool pass = b->pass_ok && b->t > 0 && n >= GROUP_STEPS;
+        if (pass && b->front_host != b->t) {
+            BCK(b, launch_set_counter(b->front + b->cur, b->t, b->stream), "step counter");
+            b->front_host = b->t;
+            b->launches += 1;
+        }
+        if (pass && n < BATCH_GRAPH_PASSES[1] * GROUP_STEPS) {
+            BCK(b, launch_pass(b, b->cur), "batch pass launch");
+            b->cur = 1 - b->cur;
+            b->t += GROUP_STEPS;
+            b->front_host = b->t;
+            n -= GROUP_STEPS;
+        } else if (pass) {
+            const int k = n >= BATCH_GRAPH_PASSES[0] * GROUP_STEPS ? 0 : 1;
+            const int lead = b->held >= 0 ? 1 : 0;
+            // the graph's first pass overwrites buffers that launched link kernels read
+            BCK(b, join_side(b), "join");
+            if (!b->pass_graph[b->cur][k][lead]) {
+                st = build_graph(b, b->cur, k, true, lead);
+                if (st != LBM_OK) return st;
+            }
+            BCK(b, cudaGraphLaunch(b->pass_graph[b->cur][k][lead], b->stream), "graph launch");
+            const int passes = BATCH_GRAPH_PASSES[k];
+            b->held = 1 - b->cur;  // an even number of passes: the last one read the other buffer
+            b->launches += ((long long)n_chunks(b) * GROUP_STEPS + 1) * passes - (1 - lead);
+            b->t += (long long)passes * GROUP_STEPS;
+            b->front_host = b->t;
+            n -= passes * GROUP_STEPS;
+        } else if (b->t == 0 || n < 2 || b->pass_ok) {
+            // the first step reads the pre-collision state; single steps run
+            // directly, after the link kernels of the passes
+            BCK(b, flush_link(b), "link launch");
+            if (b->read_live) BCK(b, join_side(b), "join");
             BCK(b, launch_step(b, b->t == 0 ? -1 : b->cur), "batch step launch");
             b->cur = 1 - b->cur;
             b->t += 1;
@@ -751,7 +946,7 @@ lbm_status lbm_batch_step(lbm_batch *b, int n)
             const int k = n >= BATCH_GRAPH_STEPS ? 0 : 1;
             const int steps = k == 0 ? BATCH_GRAPH_STEPS : 2;
             if (!b->graph[b->cur][k]) {
-                st = build_graph(b, b->cur, k);
+                st = build_graph(b, b->cur, k, false, 0);
                 if (st != LBM_OK) return st;
             }
             BCK(b, cudaGraphLaunch(b->graph[b->cur][k], b->stream), "graph launch");
@@ -760,6 +955,8 @@ lbm_status lbm_batch_step(lbm_batch *b, int n)
             n -= steps;
         }
     }
+    BCK(b, flush_link(b), "link launch");
+    BCK(b, join_side(b), "join");
     int bst[2];
     std::vector<int> dst((size_t)2 * b->n);
     BCK(b, cudaMemcpyAsync(bst, b->bstatus, sizeof(bst), cudaMemcpyDeviceToHost, b->stream), "D2H status");
@@ -858,12 +1055,15 @@ lbm_status lbm_batch_prepare(lbm_batch *b, long n)
     if (n < 0) return berr(b, LBM_EINVAL, "n must be >= 0");
     lbm_status st = ensure_series(b, b->t + n);
     if (st != LBM_OK) return st;
+    st = ensure_passes(b);
+    if (st != LBM_OK) return st;
     for (int c = 0; c < 2; ++c)
         for (int k = 0; k < 2; ++k)
-            if (!b->graph[c][k]) {
-                st = build_graph(b, c, k);
-                if (st != LBM_OK) return st;
-            }
+            for (int lead = 0; lead < (b->pass_ok ? 2 : 1); ++lead)  // a batch that takes passes replays no graph of single steps
+                if (!(b->pass_ok ? b->pass_graph[c][k][lead] : b->graph[c][k])) {
+                    st = build_graph(b, c, k, b->pass_ok, lead);
+                    if (st != LBM_OK) return st;
+                }
     return LBM_OK;
 }
 

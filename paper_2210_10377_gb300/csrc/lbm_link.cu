@@ -363,12 +363,14 @@ cudaError_t launch_link_force(int storage, const LinkGroupArgs &g, cudaStream_t 
 }
 
 // ---------------------------------------------------------------------------
-// Batched link force: one CTA per domain of a batch, the same sums and rows
-// as k_link_force.  The series holds rows [step][domain].  Every CTA reads the
-// shared step counter before it takes its ticket; the last CTA to arrive
-// advances the counter, so no CTA can see the new value.
+// Batched link force: one CTA per domain of a batch (and step, GROUP), the
+// same sums and rows as k_link_force.  The series holds rows [step][domain].
+// With several steps in the launch the last CTA of a domain to arrive
+// completes its rows in step order.  Every CTA reads the shared step counter
+// before it takes a ticket; the last domain to arrive advances the counter, so
+// no CTA can see the new value.
 // ---------------------------------------------------------------------------
-template <int S>
+template <int S, bool GROUP>
 __global__ void __launch_bounds__(BATCH_LINK_THREADS) k_link_force_batch(BatchLinkArgs b)
 {
     using A = typename AccOf<S>::type;
@@ -376,8 +378,9 @@ __global__ void __launch_bounds__(BATCH_LINK_THREADS) k_link_force_batch(BatchLi
     constexpr int WORDS = (int)(sizeof(LinkArgs) / 4);
     __shared__ LinkArgs la;
     __shared__ long long t_sh;
+    const int step = GROUP ? blockIdx.y : 0;
     {
-        const int *src = (const int *)(b.args + blockIdx.x);
+        const int *src = (const int *)(b.args + (long long)step * b.n_domains + blockIdx.x);
         int *dst = (int *)&la;
         for (int w = threadIdx.x; w < WORDS; w += BATCH_LINK_THREADS) dst[w] = src[w];
         if (threadIdx.x == 0) t_sh = *(volatile long long *)b.step_ctr;
@@ -397,47 +400,75 @@ __global__ void __launch_bounds__(BATCH_LINK_THREADS) k_link_force_batch(BatchLi
             const A tk = shfl_idx(v[k], 0);
             if (lane == k) mine = tk;
         }
-        const double dk = acc_double(mine);
-        const long long t = t_sh;
-        const long long kp = b.keep_all ? t - 1 : ((t - 1) & 1), kc = b.keep_all ? t : (t & 1);
+        double dk = acc_double(mine);
+        double *const totals = b.totals + (long long)blockIdx.x * GROUP_STEPS * 16;
+        if constexpr (GROUP) {
+            if (lane < 16) __stcg(totals + 16 * step + lane, dk);
+            __threadfence();
+            __syncwarp();
+            unsigned int last = 0;
+            if (lane == 0) last = atomicAdd(b.tickets + blockIdx.x, 1u);
+            last = __shfl_sync(0xffffffffu, last, 0);
+            if (last != (unsigned int)b.steps - 1) return;
+            __threadfence();
+            if (lane == 0) b.tickets[blockIdx.x] = 0u;
+        }
+        const int steps = GROUP ? b.steps : 1;
         const long long stride = (long long)b.n_domains * SERIES_ROW;
-        double *prev = nullptr, *cur = nullptr;
-        if (t >= 1 && la.carry[4] != 0.0) {
-            if (kp < b.series_rows)
-                prev = b.series + stride * kp + SERIES_ROW * (long long)blockIdx.x;
-            else if (lane == 0)
-                atomicOr(b.status, 4);
+        for (int j = 0; j < steps; ++j) {
+            if constexpr (GROUP) dk = __ldcg(totals + 16 * j + (lane & 15));
+            const long long t = t_sh + j;
+            const long long kp = b.keep_all ? t - 1 : ((t - 1) & 1), kc = b.keep_all ? t : (t & 1);
+            double *prev = nullptr, *cur = nullptr;
+            if (t >= 1 && la.carry[4] != 0.0) {
+                if (kp < b.series_rows)
+                    prev = b.series + stride * kp + SERIES_ROW * (long long)blockIdx.x;
+                else if (lane == 0)
+                    atomicOr(b.status, 4);
+            }
+            if (!b.drtt_only) {
+                if (kc < b.series_rows)
+                    cur = b.series + stride * kc + SERIES_ROW * (long long)blockIdx.x;
+                else if (lane == 0)
+                    atomicOr(b.status, 4);
+            }
+            finish_rows_warp(la, dk, t, prev, cur, b.drtt_only != 0);
+            __syncwarp();
         }
-        if (!b.drtt_only) {
-            if (kc < b.series_rows)
-                cur = b.series + stride * kc + SERIES_ROW * (long long)blockIdx.x;
-            else if (lane == 0)
-                atomicOr(b.status, 4);
-        }
-        finish_rows_warp(la, dk, t, prev, cur, b.drtt_only != 0);
         __threadfence();
         __syncwarp();
         if (lane == 0) {
             const unsigned int ticket = atomicAdd(b.ticket, 1u);
             if (ticket == gridDim.x - 1) {
                 *b.ticket = 0u;
-                if (!b.drtt_only) *b.step_ctr = t + 1;
+                if (!b.drtt_only) *b.step_ctr = t_sh + steps;
             }
         }
     }
 }
 
-cudaError_t launch_link_force_batch(int storage, const BatchLinkArgs &b, cudaStream_t st)
+cudaError_t launch_link_force_batch(int storage, const BatchLinkArgs &b, cudaStream_t st, int priority)
 {
-    const int grid = b.n_domains;
-    if (grid < 1) return cudaSuccess;
+    if (b.n_domains < 1) return cudaSuccess;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributePriority;
+    attr[0].val.priority = priority;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(b.n_domains, b.steps);
+    cfg.blockDim = dim3(BATCH_LINK_THREADS);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = priority != 0 ? 1 : 0;
+    const bool group = b.steps > 1;
     switch (storage) {
-    case LBM_F64: k_link_force_batch<LBM_F64><<<grid, BATCH_LINK_THREADS, 0, st>>>(b); break;
-    case LBM_F32: k_link_force_batch<LBM_F32><<<grid, BATCH_LINK_THREADS, 0, st>>>(b); break;
-    case LBM_F32_DEV: k_link_force_batch<LBM_F32_DEV><<<grid, BATCH_LINK_THREADS, 0, st>>>(b); break;
-    default: k_link_force_batch<LBM_F16_DEV><<<grid, BATCH_LINK_THREADS, 0, st>>>(b); break;
+#define GBLBM_LB(S) \
+    (group ? cudaLaunchKernelEx(&cfg, k_link_force_batch<S, true>, b) : cudaLaunchKernelEx(&cfg, k_link_force_batch<S, false>, b))
+    case LBM_F64: return GBLBM_LB(LBM_F64);
+    case LBM_F32: return GBLBM_LB(LBM_F32);
+    case LBM_F32_DEV: return GBLBM_LB(LBM_F32_DEV);
+    default: return GBLBM_LB(LBM_F16_DEV);
+#undef GBLBM_LB
     }
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
