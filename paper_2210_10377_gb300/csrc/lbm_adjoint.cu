@@ -30,7 +30,7 @@ struct AdjArgs {
     const uint8_t *tile_flag;  // per collide-stream tile: 0 = every node's bits are 0 (or NULL)
     const double *u_row;
     double *du_acc;        // [ny] running dJ/du_in
-    double *dw_acc;        // [blocks * ADJ_WARPS] running per-warp dJ/domega: FP64, or a
+    double *dw_acc;        // [blocks * warps] running per-warp dJ/domega: FP64, or a
                            // float-float pair in the same 8 bytes below FP64 storage
     long long plane;
     int nx, ny, pitch;
@@ -54,17 +54,32 @@ __device__ __forceinline__ T lam_fold(const T *__restrict__ lam, long long plane
     return v;
 }
 
-// Tiles of the backward step: 128 nodes along x by ADJ_TR rows, ADJ_RPT rows
-// a thread (all loads of a thread issued before its arithmetic).
-constexpr int ADJ_TX = 128, ADJ_TR = 4, ADJ_RPT = 2;
-constexpr int ADJ_THREADS = ADJ_TX * (ADJ_TR / ADJ_RPT);
-constexpr int ADJ_WARPS = ADJ_THREADS / 32;
-
-// Minimum resident CTAs per SM asked of the compiler (a tuning knob: 4 CTAs
-// of 256 threads, 64 registers, measured fastest of 0, 3 and 4).
-#ifndef GBLBM_ADJ_MINB
-#define GBLBM_ADJ_MINB 4
-#endif
+// Tiles of the backward step: 128 nodes along x by TR rows, RPT rows a thread
+// (all loads of a thread issued before its arithmetic), at least MINB resident
+// CTAs an SM asked of the compiler.  Large grids, bound by HBM and latency: 4
+// rows by two a thread, 4 CTAs of 256 threads with 64 registers (measured
+// fastest of 0, 3 and 4 CTAs, of one row a thread and of 2- and 8-row tiles:
+// 268 us a forward and backward step at 4096 x 2048 FP32 against 275-316).
+// Small grids, whose CTAs all fit the GPU at once, are one chain of latencies:
+// one row a thread in 2-row tiles, launched early (AdjSmall; 512 x 256 FP32:
+// 18.3 -> 15.3 us).
+constexpr int ADJ_TX = 128;
+struct AdjLarge {
+    static constexpr int TR = 4, RPT = 2, MINB = 4;
+    static constexpr bool EARLY = false;
+};
+struct AdjSmall {
+    static constexpr int TR = 2, RPT = 1, MINB = 4;
+    static constexpr bool EARLY = true;
+};
+template <typename G> __host__ __device__ constexpr int adj_threads() { return ADJ_TX * (G::TR / G::RPT); }
+template <typename G> __host__ __device__ constexpr int adj_warps() { return adj_threads<G>() / 32; }
+// Whether the large form's CTAs all fit the GPU at once.
+bool adj_is_small(int nx, int ny, int sms)
+{
+    const long long ctas = (long long)((nx + ADJ_TX - 1) / ADJ_TX) * ((ny + AdjLarge::TR - 1) / AdjLarge::TR);
+    return ctas <= (long long)AdjLarge::MINB * sms;
+}
 
 // The inputs of one node of the backward step: lt = lambda(t+1) gathered
 // along the transposed streaming (L = lambda(t+1) folded at the outlet, bounce-
@@ -185,7 +200,7 @@ __device__ __forceinline__ typename Traits<S>::comp_t adj_node(const AdjArgs &a,
 // y0-1 .. y0+TR of all nine planes, one bulk prefetch per plane and row, each
 // inside its buffer (row in [0, ny), columns x0 .. min(x0 + 128, pitch) - 1)
 // and on a 16-byte boundary (pitch is a multiple of 64 elements).
-template <int S>
+template <int S, int ADJ_TR>
 __device__ __forceinline__ void adj_prefetch(const AdjArgs &a)
 {
     using T = typename Traits<S>::comp_t;
@@ -208,15 +223,18 @@ __device__ __forceinline__ void adj_prefetch(const AdjArgs &a)
                     (unsigned)(ncol * sizeof(T)));
 }
 
-template <int S>
-__global__ void __launch_bounds__(ADJ_THREADS, GBLBM_ADJ_MINB) k_adjoint_step(AdjArgs a)
+template <int S, typename G>
+__global__ void __launch_bounds__(adj_threads<G>(), G::MINB) k_adjoint_step(AdjArgs a)
 {
+    constexpr int ADJ_TR = G::TR, ADJ_RPT = G::RPT, ADJ_WARPS = adj_warps<G>();
     using T = typename Traits<S>::comp_t;
     using Acc = typename AccOf<S>::type;
-    constexpr int ADJ_FLAGS = ADJ_TR / tile_rows(S);  // collide-stream tiles in a tile of this kernel
-    static_assert(ADJ_TR % tile_rows(S) == 0, "whole collide-stream tiles");
+    // collide-stream tile rows that a tile of this kernel meets
+    constexpr int ADJ_FLAGS = ADJ_TR > tile_rows(S) ? ADJ_TR / tile_rows(S) : 1;
+    static_assert(ADJ_TR % tile_rows(S) == 0 || tile_rows(S) % ADJ_TR == 0, "tiles in whole tiles");
+    if constexpr (G::EARLY) asm volatile("griddepcontrol.launch_dependents;");
     T *__restrict__ lam = (T *)a.lam;
-    adj_prefetch<S>(a);
+    if constexpr (!G::EARLY) adj_prefetch<S, ADJ_TR>(a);
     const int x = blockIdx.x * ADJ_TX + threadIdx.x;
     const int y0 = blockIdx.y * ADJ_TR + threadIdx.y * ADJ_RPT;
     // a tile whose nodes all have zero bits (no solid in or next to it) skips
@@ -225,8 +243,8 @@ __global__ void __launch_bounds__(ADJ_THREADS, GBLBM_ADJ_MINB) k_adjoint_step(Ad
     if (plain_tile) {
 #pragma unroll
         for (int k = 0; k < ADJ_FLAGS; ++k) {
-            const int ty = (int)blockIdx.y * ADJ_FLAGS + k;
-            if (ty * (ADJ_TR / ADJ_FLAGS) < a.ny && a.tile_flag[(long long)ty * gridDim.x + blockIdx.x]) plain_tile = false;
+            const int ty = (int)blockIdx.y * ADJ_TR / tile_rows(S) + k;
+            if (ty * tile_rows(S) < a.ny && a.tile_flag[(long long)ty * gridDim.x + blockIdx.x]) plain_tile = false;
         }
     }
     Acc dw;
@@ -240,6 +258,8 @@ __global__ void __launch_bounds__(ADJ_THREADS, GBLBM_ADJ_MINB) k_adjoint_step(Ad
             const int y = y0 + r;
             nb[r] = (plain_tile || y >= a.ny) ? (uint16_t)0 : a.nbits[(long long)y * a.pitch + x];
         }
+        // the step before has to be done before its lambda is read
+        if constexpr (G::EARLY) asm volatile("griddepcontrol.wait;" ::: "memory");
 #pragma unroll
         for (int r = 0; r < ADJ_RPT; ++r) {
             const int y = y0 + r;
@@ -271,6 +291,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, GBLBM_ADJ_MINB) k_adjoint_step(Ad
             }
         }
     }
+    if constexpr (G::EARLY) asm volatile("griddepcontrol.wait;" ::: "memory");  // threads past the grid, too
     // running sums of dJ/domega, one slot per warp (fixed order within the
     // warp; float-float below FP64 storage, the running slot included, so
     // that no FP64 instruction runs per step, and no barrier between warps)
@@ -301,9 +322,33 @@ __global__ void __launch_bounds__(256) k_sum_fixed(const A *__restrict__ v, long
 }
 
 // slots of the per-warp dJ/domega sums
-int adjoint_blocks(int nx, int ny)
+int adjoint_blocks(int nx, int ny, int sm_count)
 {
-    return ((nx + ADJ_TX - 1) / ADJ_TX) * ((ny + ADJ_TR - 1) / ADJ_TR) * ADJ_WARPS;
+    const bool small = adj_is_small(nx, ny, sm_count);
+    const int tr = small ? AdjSmall::TR : AdjLarge::TR;
+    return ((nx + ADJ_TX - 1) / ADJ_TX) * ((ny + tr - 1) / tr) * (small ? adj_warps<AdjSmall>() : adj_warps<AdjLarge>());
+}
+
+template <typename G>
+cudaError_t adj_launch(int storage, const AdjArgs &a, dim3 grid, bool follows, cudaStream_t st)
+{
+    // An early launch (see launch_collide_stream): the CTAs load their
+    // neighbour bits while the step before drains.
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(ADJ_TX, G::TR / G::RPT);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = G::EARLY && follows ? 1 : 0;
+    switch (storage) {
+    case LBM_F64: return cudaLaunchKernelEx(&cfg, k_adjoint_step<LBM_F64, G>, a);
+    case LBM_F32: return cudaLaunchKernelEx(&cfg, k_adjoint_step<LBM_F32, G>, a);
+    case LBM_F32_DEV: return cudaLaunchKernelEx(&cfg, k_adjoint_step<LBM_F32_DEV, G>, a);
+    default: return cudaLaunchKernelEx(&cfg, k_adjoint_step<LBM_F16_DEV, G>, a);
+    }
 }
 
 cudaError_t launch_adjoint_step(int storage, const void *src, int precollision, const void *lam_next, void *lam,
@@ -311,7 +356,7 @@ cudaError_t launch_adjoint_step(int storage, const void *src, int precollision, 
                                 const double *u_row, double *du_acc,
                                 double *dw_acc, long long plane, int nx, int ny, int pitch,
                                 int in_window, double omega, double rho0, double obj_x,
-                                double obj_y, cudaStream_t st)
+                                double obj_y, bool follows, cudaStream_t st)
 {
     AdjArgs a;
     a.src = src;
@@ -335,34 +380,36 @@ cudaError_t launch_adjoint_step(int storage, const void *src, int precollision, 
         a.obj[i] = obj_x * cx(i) + obj_y * cy(i);
         a.obj_f[i] = (float)a.obj[i];
     }
-    dim3 grid((nx + ADJ_TX - 1) / ADJ_TX, (ny + ADJ_TR - 1) / ADJ_TR);
-    dim3 block(ADJ_TX, ADJ_TR / ADJ_RPT);
-    // the collide-stream tile flags serve when whole ones make up these tiles
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        cudaGetLastError();
+    const bool small = adj_is_small(nx, ny, sms);
+    const int tr = small ? AdjSmall::TR : AdjLarge::TR;
+    const dim3 grid((nx + ADJ_TX - 1) / ADJ_TX, (ny + tr - 1) / tr);
+    // the collide-stream tile flags serve when they are as wide as these tiles
     a.tile_flag = (tile_flag && TILE_X == ADJ_TX && flag_rows == tile_rows(storage) && flag_tiles_x == (int)grid.x)
                       ? tile_flag
                       : nullptr;
+    if (small) {
+        a.pf_rows = 0;
+        return adj_launch<AdjSmall>(storage, a, grid, follows, st);
+    }
     // prefetch half the CTAs the GPU holds at once ahead, in tile rows
     int pf_rows = 0;
     if (storage != LBM_F64) {
-        int dev = 0, sms = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const void *fn = storage == LBM_F32 ? (const void *)k_adjoint_step<LBM_F32>
-                         : storage == LBM_F32_DEV ? (const void *)k_adjoint_step<LBM_F32_DEV>
-                                                  : (const void *)k_adjoint_step<LBM_F16_DEV>;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, ADJ_THREADS, 0) == cudaSuccess && sms > 0)
+        int per_sm = 0;
+        const void *fn = storage == LBM_F32       ? (const void *)k_adjoint_step<LBM_F32, AdjLarge>
+                         : storage == LBM_F32_DEV ? (const void *)k_adjoint_step<LBM_F32_DEV, AdjLarge>
+                                                  : (const void *)k_adjoint_step<LBM_F16_DEV, AdjLarge>;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, adj_threads<AdjLarge>(), 0) == cudaSuccess &&
+            sms > 0)
             pf_rows = (int)(((long long)per_sm * sms / 2 + grid.x / 2) / grid.x);
         cudaGetLastError();
         if (pf_rows < 1) pf_rows = 1;
     }
     a.pf_rows = pf_rows;
-    switch (storage) {
-    case LBM_F64: k_adjoint_step<LBM_F64><<<grid, block, 0, st>>>(a); break;
-    case LBM_F32: k_adjoint_step<LBM_F32><<<grid, block, 0, st>>>(a); break;
-    case LBM_F32_DEV: k_adjoint_step<LBM_F32_DEV><<<grid, block, 0, st>>>(a); break;
-    default: k_adjoint_step<LBM_F16_DEV><<<grid, block, 0, st>>>(a); break;
-    }
-    return cudaGetLastError();
+    return adj_launch<AdjLarge>(storage, a, grid, follows, st);
 }
 
 cudaError_t launch_sum_fixed(const double *v, long long n, double *out, bool ff_slots, cudaStream_t st)

@@ -488,6 +488,7 @@ cudaError_t launch_one_pass(lbm_ctx *h, int src)
             a.partials = pass_partials(h, src, j);
             a.step_ctr = h->front + src;
             a.step_off = j;
+        a.pass = 1;
             a.next_ctr = j == 0 ? h->front + dst : nullptr;
             a.early = j > 0 && h->tiles_x * h->tiles_y <= EARLY_CTAS * h->sm_count;
             e = launch_collide_stream(h->storage, a, h->tiles_x, h->tiles_y, false, nullptr, h->stream);
@@ -1070,6 +1071,42 @@ lbm_status queue_steps(lbm_ctx *h, int n)
     return LBM_OK;
 }
 
+// GROUP_STEPS eager steps from state j of `slots` on, for queue_steps_keep:
+// the collide-stream kernels in turn, then one link kernel for them on the
+// side stream.  set: which control-volume slices and step counter they use
+// (each group the next of NBUF).
+cudaError_t launch_kept_group(lbm_ctx *h, const void *const *state, int set)
+{
+    cudaError_t e = h->ev_live[set] ? cudaStreamWaitEvent(h->stream, h->ev_read[set], 0) : cudaSuccess;
+    LinkGroupArgs g = link_group(h, link_args(h, h->cur, next_buf(h->cur), 0, 0));
+    g.steps = GROUP_STEPS;
+    for (int j = 0; j <= GROUP_STEPS; ++j) {
+        g.state[j] = state[j];
+        g.plane[j] = h->plane;
+    }
+    for (int j = 0; j < GROUP_STEPS && e == cudaSuccess; ++j) {
+        StepArgs a = step_args(h, h->cur, next_buf(h->cur), 0);
+        a.src = state[j];
+        a.dst = const_cast<void *>(state[j + 1]);
+        a.partials = pass_partials(h, set, j);
+        g.partials[j] = a.partials;
+        a.step_ctr = h->front + set;
+        a.step_off = j;
+        a.pass = 1;
+        a.next_ctr = j == 0 ? h->front + next_buf(set) : nullptr;
+        a.early = j > 0 && h->tiles_x * h->tiles_y <= EARLY_CTAS * h->sm_count;
+        e = launch_collide_stream(h->storage, a, h->tiles_x, h->tiles_y, false, nullptr, h->stream);
+        h->launches += 1;
+    }
+    if (e == cudaSuccess) e = cudaEventRecord(h->ev_fork, h->stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->ev_fork, 0);
+    if (e == cudaSuccess) e = launch_link_force(h->storage, g, h->side, h->link_prio);
+    if (e == cudaSuccess) e = cudaEventRecord(h->ev_read[set], h->side);
+    h->ev_live[set] = true;
+    h->launches += 1;
+    return e;
+}
+
 // Queues n eager steps whose states are kept for a backward sweep: step j
 // (0-based) reads slot j and writes slot j + 1 of `slots` (stride bytes
 // apart; slot 0 holds a copy of the current state), except the last step,
@@ -1077,26 +1114,52 @@ lbm_status queue_steps(lbm_ctx *h, int n)
 // buffer it writes at its slot, so the kernels, the held link kernels and the
 // force series are exactly those of queue_steps; only the population
 // addresses differ.  The direct collide-stream kernel serves these steps (the
-// staged kernel's tensor maps describe the handle's own buffers).
+// staged kernel's tensor maps describe the handle's own buffers).  Grids that
+// take passes of single steps take their link kernels in groups here, too.
 lbm_status queue_steps_keep(lbm_ctx *h, int n, char *slots, size_t stride)
 {
     lbm_status st = ensure_series(h, h->t + n);
     if (st == LBM_OK) st = arm_status(h);
     if (st != LBM_OK) return st;
+    if (n > GROUP_STEPS) ensure_passes(h);
+    const bool groups = h->pass_kind == PASS_STEPS;
     void *orig[NBUF];
     for (int b = 0; b < NBUF; ++b) orig[b] = h->pop[b];
-    const int bulk = h->use_bulk;
+    const int bulk = h->use_bulk, end = (h->cur + n) % NBUF;  // the buffer of the last state
     h->use_bulk = 0;
     cudaError_t e = cudaSuccess;
-    for (int j = 0; j < n && e == cudaSuccess; ++j) {
+    auto state = [&](int j) { return j < n ? (void *)(slots + (size_t)j * stride) : orig[end]; };
+    bool counted = false;
+    for (int j = 0; j < n && e == cudaSuccess;) {
+        if (groups && !h->precollision && n - j >= GROUP_STEPS) {
+            const int set = h->cur;  // GROUP_STEPS = NBUF + 1: each group starts on the next buffer
+            static_assert(GROUP_STEPS % NBUF == 1, "groups take the counters and slices in turn");
+            e = flush_link(h);
+            if (e == cudaSuccess && !counted) {
+                e = join_side(h);
+                if (e == cudaSuccess) e = launch_set_counter(h->front + set, h->t, h->stream);
+                h->front_host = -1;
+                counted = true;
+            }
+            const void *states[GROUP_STEPS + 1];
+            for (int k = 0; k <= GROUP_STEPS; ++k) states[k] = state(j + k);
+            if (e == cudaSuccess) e = launch_kept_group(h, states, set);
+            j += GROUP_STEPS;
+            h->cur = (h->cur + GROUP_STEPS) % NBUF;
+            h->pop[h->cur] = state(j);
+            h->t += GROUP_STEPS;
+            if (n - j < GROUP_STEPS && e == cudaSuccess) e = join_side(h);  // single steps follow, or the end
+            continue;
+        }
         const int db = next_buf(h->cur);
         // the held link kernel of step j-1 reads buffers prev(cur) and cur,
         // whose addresses stay as they were
-        h->pop[db] = j + 1 < n ? (void *)(slots + (size_t)(j + 1) * stride) : orig[db];
+        h->pop[db] = state(j + 1);
         e = launch_one_step(h, h->cur, h->precollision, nullptr);
         h->cur = db;
         h->precollision = 0;
         h->t += 1;
+        ++j;
     }
     if (e == cudaSuccess) e = flush_link(h);
     if (e == cudaSuccess) e = join_side(h);
@@ -1466,7 +1529,7 @@ lbm_status lbm_adjoint(lbm_ctx *h, int steps, int window, double wx, double wy, 
     const size_t buf_bytes = 9 * (size_t)h->plane * h->elem;
     const size_t comp = h->storage == LBM_F64 ? 8 : 4;
     const size_t comp_bytes = 9 * (size_t)h->plane * comp;
-    const int nblk = adjoint_blocks(h->nx, h->ny);
+    const int nblk = adjoint_blocks(h->nx, h->ny, h->sm_count);
     cudaStream_t st = h->stream;
     auto isqrt_up = [](long long n) {
         long long k = 1;
@@ -1595,7 +1658,7 @@ lbm_status lbm_adjoint(lbm_ctx *h, int steps, int window, double wx, double wy, 
         e = launch_adjoint_step(h->storage, keep + buf_bytes * (size_t)j, j == 0 ? keep_pre : 0, lam_next, lam_cur,
                                 h->nbits, h->tile_flag, tile_rows(h->storage), h->tiles_x, h->u_row, du_acc, dw_acc,
                                 h->plane, h->nx, h->ny, h->pitch, t >= steps - window, h->omega, h->rho0, obj_x,
-                                obj_y, st);
+                                obj_y, j < L - 1, st);
         char *tmp = lam_next;
         lam_next = lam_cur;
         lam_cur = tmp;
@@ -1620,7 +1683,7 @@ lbm_status lbm_adjoint(lbm_ctx *h, int steps, int window, double wx, double wy, 
             e = launch_adjoint_step(h->storage, state(s), s == 0 ? ckpre[k] : 0, lam_next, lam_cur, h->nbits,
                                     h->tile_flag, tile_rows(h->storage), h->tiles_x, h->u_row, du_acc, dw_acc,
                                     h->plane, h->nx, h->ny, h->pitch,
-                                    t >= steps - window, h->omega, h->rho0, obj_x, obj_y, st);
+                                    t >= steps - window, h->omega, h->rho0, obj_x, obj_y, s < n - 1, st);
             char *tmp = lam_next;
             lam_next = lam_cur;
             lam_cur = tmp;

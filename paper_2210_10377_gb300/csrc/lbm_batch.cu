@@ -82,7 +82,7 @@ __device__ __forceinline__ void batch_tile(const BatchParams &p, int k)
         a.use_bulk = 0;
         a.sm_count = 0;
         a.step_off = p.step_off;
-        a.early = 0;
+        a.pass = a.early = 0;
         a.next_ctr = nullptr;
         collide_tile<S, MOMENTUM_ONLY, false, TX, TR, RPT>(a, e.y, e.z, p.precollision || e.w != 0);
     }

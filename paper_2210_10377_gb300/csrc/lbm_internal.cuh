@@ -163,6 +163,7 @@ struct StepArgs {
     int first_r0, first_r1;  // tile rows with bounce-back tiles, dispatched first (r0 > r1: none)
     unsigned int wait_limit; // polls of each pipeline wait of the staged kernel (WAIT_LIMIT)
     int step_off;            // this launch's step is *step_ctr + step_off
+    int pass;                // a step of a pass (step_off, early, next_ctr may be set)
     int early;               // launched while its predecessor may still run (see launch_collide_stream)
     long long *next_ctr;     // receives *step_ctr + GROUP_STEPS (NULL: nothing): the counter of the next pass
 };
@@ -276,7 +277,8 @@ cudaError_t launch_scatter_pop(int storage, void *pop, const uint16_t *nbits, lo
 
 // discrete adjoint (lbm_adjoint.cu): one backward step; src holds ft(t-1) in
 // the storage type (f(t) itself when precollision), pulled inside the kernel
-int adjoint_blocks(int nx, int ny);
+int adjoint_blocks(int nx, int ny, int sm_count);
+// follows: the launch before it on the stream is a backward step
 // tile_flag: the collide-stream tile flags (tiles of TILE_X x flag_rows nodes,
 // flag_tiles_x a row), used when they match the backward step's tiles
 cudaError_t launch_adjoint_step(int storage, const void *src, int precollision, const void *lam_next, void *lam,
@@ -284,7 +286,7 @@ cudaError_t launch_adjoint_step(int storage, const void *src, int precollision, 
                                 const double *u_row, double *du_acc,
                                 double *dw_acc, long long plane, int nx, int ny, int pitch,
                                 int in_window, double omega, double rho0, double obj_x,
-                                double obj_y, cudaStream_t st);
+                                double obj_y, bool follows, cudaStream_t st);
 // sum of n slots in a fixed order: FP64 values, or float-float pairs (ff_slots)
 cudaError_t launch_sum_fixed(const double *v, long long n, double *out, bool ff_slots, cudaStream_t st);
 // lambda (compute type, [9][ny][pitch]) -> dJ/df0 in FP64 [9][ny][nx] in device

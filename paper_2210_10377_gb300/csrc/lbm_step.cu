@@ -99,21 +99,28 @@ __device__ __forceinline__ void prefetch_ahead(const StepArgs &a)
 // Direct-load collide-stream kernel: one CTA of 128 x (TR/RPT) threads per
 // 128 x TR tile; tiles without solids away from the domain's edges take the
 // interior path (collide_tile).
-template <int S, bool MOMENTUM_ONLY, bool FORCE>
+// PASS: a step of a pass, which may be launched early (StepArgs::early, see
+// launch_collide_stream) and whose first step sets the next pass's counter;
+// apart, because what it does first costs a large grid 6 % (4096 x 2048 FP32:
+// 91.7 -> 97.8 us a launch).
+template <int S, bool MOMENTUM_ONLY, bool FORCE, bool PASS>
 __global__ void __launch_bounds__((TILE_X / cols_per_thread(S)) * (tile_rows(S) / direct_rpt(S)),
                                   DirectMinBlocks<S>::value)
     k_collide_stream(StepArgs a)
 {
-    // the next step's CTAs may be placed; they wait here for this grid's end
-    // before they read or write anything this one does
-    if constexpr (!MOMENTUM_ONLY) asm volatile("griddepcontrol.launch_dependents;");
+    if constexpr (PASS)
+        // the next step's CTAs may be placed; they wait for this grid's end
+        // before they read or write anything that it does
+        asm volatile("griddepcontrol.launch_dependents;");
+    else if constexpr (!MOMENTUM_ONLY)
+        prefetch_ahead<S>(a);
+    // a launch over a sub-rectangle of tiles (the momentum-only pass) keeps plain order
     const int tx = blockIdx.x + a.tile_off_x;
     const int ty = (MOMENTUM_ONLY || a.tile_off_y != 0) ? (int)blockIdx.y + a.tile_off_y
                                                         : tile_row_of((int)blockIdx.y, (int)gridDim.y,
                                                                       a.first_r0, a.first_r1);
-    // a launch over a sub-rectangle of tiles (the momentum-only pass) keeps plain order
     const bool checked = a.precollision || a.tile_flag[(long long)ty * a.tiles_x + tx] != 0;
-    if constexpr (!MOMENTUM_ONLY) {
+    if constexpr (PASS) {
         if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
         prefetch_ahead<S>(a);
         if (a.next_ctr && (blockIdx.x | blockIdx.y | threadIdx.x | threadIdx.y) == 0)
@@ -357,13 +364,13 @@ int collide_stream_prefetch_rows(int storage, int sm_count, int tiles_x)
     cudaError_t e;
     switch (storage) {
     case LBM_F32:
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_collide_stream<LBM_F32, false, false>, threads, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_collide_stream<LBM_F32, false, false, false>, threads, 0);
         break;
     case LBM_F32_DEV:
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_collide_stream<LBM_F32_DEV, false, false>, threads, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_collide_stream<LBM_F32_DEV, false, false, false>, threads, 0);
         break;
     default:
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_collide_stream<LBM_F16_DEV, false, false>, threads, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_collide_stream<LBM_F16_DEV, false, false, false>, threads, 0);
         break;
     }
     if (e != cudaSuccess) {
@@ -405,9 +412,11 @@ cudaError_t launch_collide_stream(int storage, const StepArgs &a, int tiles_x, i
     cfg.attrs = attr;
     cfg.numAttrs = a.early ? 1 : 0;
 #define GBLBM_CS(S)                                                                                       \
-    return momentum_only ? cudaLaunchKernelEx(&cfg, k_collide_stream<S, true, false>, a)                  \
-           : force       ? cudaLaunchKernelEx(&cfg, k_collide_stream<S, false, true>, a)                  \
-                         : cudaLaunchKernelEx(&cfg, k_collide_stream<S, false, false>, a)
+    return momentum_only ? cudaLaunchKernelEx(&cfg, k_collide_stream<S, true, false, false>, a)           \
+           : a.pass      ? (force ? cudaLaunchKernelEx(&cfg, k_collide_stream<S, false, true, true>, a)   \
+                                  : cudaLaunchKernelEx(&cfg, k_collide_stream<S, false, false, true>, a)) \
+           : force       ? cudaLaunchKernelEx(&cfg, k_collide_stream<S, false, true, false>, a)           \
+                         : cudaLaunchKernelEx(&cfg, k_collide_stream<S, false, false, false>, a)
     switch (storage) {
     case LBM_F64: GBLBM_CS(LBM_F64);
     case LBM_F32: GBLBM_CS(LBM_F32);
