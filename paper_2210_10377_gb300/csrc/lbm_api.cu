@@ -330,6 +330,15 @@ LinkGroupArgs link_group(lbm_ctx *h, const LinkArgs &a)
     return g;
 }
 
+// A step of a pass leaves the control-volume sums to k_cv_sums, beside the
+// link kernel: in the collide-stream kernel they lengthen the box's tiles, the
+// slowest of a small grid.
+void no_box_sums(StepArgs &a)
+{
+    a.cvt[0] = a.cvt[2] = 1;
+    a.cvt[1] = a.cvt[3] = 0;
+}
+
 // Elements between two planes of an intermediate state (the kept rows).
 long long mid_plane(const lbm_ctx *h) { return (long long)(h->keep[3] - h->keep[2] + 1) * h->pitch; }
 
@@ -394,10 +403,8 @@ cudaError_t launch_link_side(lbm_ctx *h, int src, int precollision, int steps)
         pass_states(h, src, g.state, g.plane);
         g.steps = steps;
         for (int j = 0; j < steps; ++j) g.partials[j] = c.partials[j] = pass_partials(h, src, j);
-        if (h->pass_kind == PASS_MARCH) {  // single steps have written their own
-            if (e == cudaSuccess) e = launch_cv_sums(h->storage, c, h->side, h->link_prio);
-            h->launches += 1;
-        }
+        if (e == cudaSuccess) e = launch_cv_sums(h->storage, c, h->side, h->link_prio);
+        h->launches += 1;
     }
     if (e == cudaSuccess) e = launch_link_force(h->storage, g, h->side, h->link_prio);
     if (e == cudaSuccess) e = cudaEventRecord(h->ev_read[src], h->side);
@@ -485,7 +492,7 @@ cudaError_t launch_one_pass(lbm_ctx *h, int src)
             StepArgs a = step_args(h, src, dst, 0);
             a.src = state[j];
             a.dst = const_cast<void *>(state[j + 1]);
-            a.partials = pass_partials(h, src, j);
+            no_box_sums(a);
             a.step_ctr = h->front + src;
             a.step_off = j;
         a.pass = 1;
@@ -1052,9 +1059,9 @@ lbm_status queue_steps(lbm_ctx *h, int n)
             h->lead_src = prev_buf(h->cur);  // units is a multiple of NBUF
             h->lead_pre = 0;
             h->lead_steps = each;
-            // the last link kernel (after a multi-step pass, the box sums, too) is held
+            // the last link kernel (a pass's with its box sums) is held
             const int own = !pass || h->pass_kind == PASS_MARCH ? 1 : GROUP_STEPS;
-            const int link = pass && h->pass_kind == PASS_MARCH ? 2 : 1;
+            const int link = pass ? 2 : 1;
             h->launches += (long long)(own + link) * units - link * (1 - lead);
             h->t += (long long)units * each;
             if (pass) h->front_host += (long long)units * each;
@@ -1080,16 +1087,19 @@ cudaError_t launch_kept_group(lbm_ctx *h, const void *const *state, int set)
     cudaError_t e = h->ev_live[set] ? cudaStreamWaitEvent(h->stream, h->ev_read[set], 0) : cudaSuccess;
     LinkGroupArgs g = link_group(h, link_args(h, h->cur, next_buf(h->cur), 0, 0));
     g.steps = GROUP_STEPS;
+    CvArgs c;
+    memset(&c, 0, sizeof(c));
+    c.s = step_args(h, h->cur, next_buf(h->cur), 0);
     for (int j = 0; j <= GROUP_STEPS; ++j) {
-        g.state[j] = state[j];
-        g.plane[j] = h->plane;
+        g.state[j] = c.state[j] = state[j];
+        g.plane[j] = c.plane[j] = h->plane;
     }
     for (int j = 0; j < GROUP_STEPS && e == cudaSuccess; ++j) {
         StepArgs a = step_args(h, h->cur, next_buf(h->cur), 0);
         a.src = state[j];
         a.dst = const_cast<void *>(state[j + 1]);
-        a.partials = pass_partials(h, set, j);
-        g.partials[j] = a.partials;
+        no_box_sums(a);
+        g.partials[j] = c.partials[j] = pass_partials(h, set, j);
         a.step_ctr = h->front + set;
         a.step_off = j;
         a.pass = 1;
@@ -1100,10 +1110,11 @@ cudaError_t launch_kept_group(lbm_ctx *h, const void *const *state, int set)
     }
     if (e == cudaSuccess) e = cudaEventRecord(h->ev_fork, h->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->ev_fork, 0);
+    if (e == cudaSuccess) e = launch_cv_sums(h->storage, c, h->side, h->link_prio);
     if (e == cudaSuccess) e = launch_link_force(h->storage, g, h->side, h->link_prio);
     if (e == cudaSuccess) e = cudaEventRecord(h->ev_read[set], h->side);
     h->ev_live[set] = true;
-    h->launches += 1;
+    h->launches += 2;
     return e;
 }
 

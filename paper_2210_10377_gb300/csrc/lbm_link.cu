@@ -33,8 +33,9 @@ namespace gblbm {
 // ---------------------------------------------------------------------------
 // NT threads share the ranges.  EARLY: a thread's first partial row is loaded
 // before the link loop, so that its latency overlaps the links' (the sums keep
-// their order).
-template <int S, int NT, bool EARLY>
+// their order).  AFTER: the kernel that writes the partial rows may still run
+// (an early launch); they are read after its end, the links before.
+template <int S, int NT, bool EARLY, bool AFTER = false>
 __device__ __forceinline__ void link_sums(const LinkArgs &a, long long k0, long long k1, int p0, int p1,
                                           typename AccOf<S>::type (&v)[LINK_PARTIAL])
 {
@@ -146,6 +147,7 @@ __device__ __forceinline__ void link_sums(const LinkArgs &a, long long k0, long 
             acc_add(v[5], ey > 0 ? sp : -sp);
         }
     }
+    if constexpr (AFTER) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (EARLY && s0 < p1) {
 #pragma unroll
         for (int k = 0; k < CV_PARTIAL; ++k) acc_add(v[6 + k], first[k]);
@@ -246,7 +248,7 @@ __global__ void __launch_bounds__(LINK_THREADS) k_link_force(const __grid_consta
         const int per_p = (a.n_partials + gridDim.x - 1) / gridDim.x;
         const int p0 = per_p * blockIdx.x;
         const int p1 = p0 + per_p < a.n_partials ? p0 + per_p : a.n_partials;
-        link_sums<S, LINK_THREADS, GBLBM_LINK_EARLY != 0>(l, k0, k1 > k0 ? k1 : k0, p0, p1 > p0 ? p1 : p0, v);
+        link_sums<S, LINK_THREADS, GBLBM_LINK_EARLY != 0 && !GROUP, GROUP>(l, k0, k1 > k0 ? k1 : k0, p0, p1 > p0 ? p1 : p0, v);
     }
     // each warp reduces its sums and writes them as one row (slot: CTA, warp);
     // no block barrier, and the last warp of a step to take a ticket sums it
@@ -341,17 +343,21 @@ cudaError_t launch_link_force(int storage, const LinkGroupArgs &g, cudaStream_t 
     // The priority travels with the launch, so that a captured graph node
     // keeps it: the link kernel runs beside a collide-stream kernel that
     // fills the GPU, and the collide-stream kernel two steps on waits for it.
-    cudaLaunchAttribute attr[1];
+    // A group's launch is a programmatic dependent of the kernel before it on
+    // the stream, the box sums: its link sums run beside that kernel.
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributePriority;
     attr[0].val.priority = priority;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(g.a.n_ctas, g.steps);
     cfg.blockDim = dim3(LINK_THREADS);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = priority != 0 ? 1 : 0;
     const bool group = g.steps > 1;
+    cfg.attrs = priority != 0 ? attr : attr + 1;
+    cfg.numAttrs = (priority != 0 ? 1 : 0) + (group ? 1 : 0);
     switch (storage) {
 #define GBLBM_LF(S) (group ? cudaLaunchKernelEx(&cfg, k_link_force<S, true>, g) : cudaLaunchKernelEx(&cfg, k_link_force<S, false>, g))
     case LBM_F64: return GBLBM_LF(LBM_F64);
