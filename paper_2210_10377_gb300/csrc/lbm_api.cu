@@ -56,7 +56,7 @@ constexpr double MARCH_KEEP_SHARE = 0.25;
 // with two link kernels in flight).  The second kind holds nine more states,
 // so it is for states of at most PASS_STATE_BYTES.
 enum PassKind { PASS_NONE = 0, PASS_MARCH, PASS_STEPS };
-constexpr double PASS_STATE_BYTES = 14e6;
+constexpr double PASS_STATE_BYTES = 40e6;
 // Steps of a pass follow one another early (StepArgs::early) up to this many
 // CTAs an SM.
 constexpr int EARLY_CTAS = 4;
@@ -134,7 +134,10 @@ struct lbm_ctx {
     double *carry = nullptr;     // [8]
     long long *step_ctr = nullptr;
     int *status = nullptr;       // [2]
-    int status_host[2] = {0, 0};  // the status words read back by settle
+    // Page-locked words that small results are read back into: settle's status
+    // words, then one series row (a copy to pageable memory is staged, and the
+    // host waits for the staging).
+    double *host_row = nullptr;
     bool status_armed = false;   // status cleared for the queued steps
     bool pending = false;        // steps queued and not yet settled
     long long t = 0;
@@ -719,6 +722,7 @@ void free_all(lbm_ctx *h)
                     h->u_row, h->inlet, h->partials, h->link_partials, h->ticket, h->series,
                     h->carry, h->step_ctr, h->status, h->mid, h->group_partials, h->march_units_d};
     for (void *p : bufs) dev_free(h, p);
+    if (h->host_row) cudaFreeHost(h->host_row);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
 
@@ -892,7 +896,11 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
     ALLOC(h->carry, double *, sizeof(double) * 8);
     ALLOC(h->step_ctr, long long *, sizeof(long long) * (1 + NBUF));
     h->front = h->step_ctr + 1;
-    ALLOC(h->status, int *, sizeof(int) * 2);
+    ALLOC(h->status, int *, sizeof(int) * 4);
+    if (cudaHostAlloc((void **)&h->host_row, sizeof(double) * (2 + SERIES_ROW), cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(set_err(h, LBM_ENOMEM, "allocation of page-locked memory failed"));
+    }
     st = ensure_series(h, 1024);
     if (st != LBM_OK) return fail(st);
 
@@ -906,7 +914,7 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
     CKC(cudaMemsetAsync(h->ticket, 0, sizeof(unsigned int) * 16, s), "memset");
     CKC(cudaMemsetAsync(h->carry, 0, sizeof(double) * 8, s), "memset");
     CKC(cudaMemsetAsync(h->step_ctr, 0, sizeof(long long) * (1 + NBUF), s), "memset");
-    const int status0[2] = {0, INT_MAX};
+    const int status0[4] = {0, INT_MAX, 0, INT_MAX};  // the words, and what resets them
     CKC(cudaMemcpyAsync(h->status, status0, sizeof(status0), cudaMemcpyHostToDevice, s), "H2D status");
     h->status_armed = true;
     CKC(cudaMemcpyAsync(h->mask_d, mask, N, cudaMemcpyHostToDevice, s), "H2D mask");
@@ -994,13 +1002,13 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
 namespace {
 
 // Clears the status words for the steps about to be queued, unless the last
-// settle already did: status[0] = 0 (no flag), status[1] = 0x7f7f7f7f (no bad
+// settle already did: status[0] = 0 (no flag), status[1] = INT_MAX (no bad
 // step yet).
 lbm_status arm_status(lbm_ctx *h)
 {
     if (h->status_armed) return LBM_OK;
-    CK(h, cudaMemsetAsync(h->status, 0, sizeof(int), h->stream), "status reset");
-    CK(h, cudaMemsetAsync(h->status + 1, 0x7f, sizeof(int), h->stream), "status reset");
+    CK(h, cudaMemcpyAsync(h->status, h->status + 2, 2 * sizeof(int), cudaMemcpyDeviceToDevice, h->stream),
+       "status reset");
     h->status_armed = true;
     return LBM_OK;
 }
@@ -1017,6 +1025,22 @@ lbm_status queue_steps(lbm_ctx *h, int n)
         h->events.resize(3 * TIMING_BATCH, nullptr);
         for (auto &e : h->events)
             if (!e) CK(h, cudaEventCreate(&e), "event create");
+    }
+    if (n == 1 && !h->timing && h->lead_src < 0) {
+        // a single step has nothing to run its link kernel beside: both go to
+        // the handle's stream, without the events of a fork and a join
+        const int dst = next_buf(h->cur);
+        CK(h, launch_collide_stream(h->storage, step_args(h, h->cur, dst, h->precollision), h->tiles_x, h->tiles_y,
+                                    false, h->tmap_ok ? (const void *)&h->tmap[h->cur] : nullptr, h->stream),
+           "step launch");
+        CK(h, launch_link_force(h->storage, link_group(h, link_args(h, h->cur, dst, h->precollision, 0)), h->stream),
+           "link launch");
+        h->launches += 2;
+        h->cur = dst;
+        h->precollision = 0;
+        h->t += 1;
+        h->pending = true;
+        return LBM_OK;
     }
     int nev = 0;
     if (n >= GROUP_STEPS) ensure_passes(h);
@@ -1188,14 +1212,13 @@ lbm_status settle(lbm_ctx *h)
     if (!h->pending) return LBM_OK;
     h->pending = false;
     h->status_armed = false;
-    CK(h, cudaMemcpyAsync(h->status_host, h->status, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream),
-       "D2H status");
+    CK(h, cudaMemcpyAsync(h->host_row, h->status, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream), "D2H status");
     // clear the words for the next queue here, so that its start waits on nothing
-    CK(h, cudaMemsetAsync(h->status, 0, sizeof(int), h->stream), "status reset");
-    CK(h, cudaMemsetAsync(h->status + 1, 0x7f, sizeof(int), h->stream), "status reset");
+    CK(h, cudaMemcpyAsync(h->status, h->status + 2, 2 * sizeof(int), cudaMemcpyDeviceToDevice, h->stream),
+       "status reset");
     CK(h, cudaStreamSynchronize(h->stream), "step sync");
     h->status_armed = true;
-    const int *status = h->status_host;
+    const int status[2] = {((const int *)h->host_row)[0], ((const int *)h->host_row)[1]};
     if (h->t - 1 > h->carry_from) h->drtt_ready = h->t - 1 > h->drtt_ready ? h->t - 1 : h->drtt_ready;
     if (status[0] & 4)
         return set_err(h, LBM_ESTATE, "a force-series row lay beyond the series buffer");
@@ -1254,6 +1277,16 @@ lbm_status lbm_force_series(lbm_ctx *h, int scheme, long first, long count, doub
         if (st != LBM_OK) return st;
     }
     const size_t R = SERIES_ROW;
+    if (count == 1) {
+        double *row = h->host_row + 2;
+        CK(h, cudaMemcpyAsync(row, h->series + R * (h->record_series ? first : (first & 1)), sizeof(double) * R,
+                              cudaMemcpyDeviceToHost, h->stream),
+           "D2H series");
+        CK(h, cudaStreamSynchronize(h->stream), "sync");
+        fx[0] = row[2 * scheme];
+        fy[0] = row[2 * scheme + 1];
+        return LBM_OK;
+    }
     std::vector<double> rows((size_t)count * R);
     if (h->record_series) {
         CK(h, cudaMemcpyAsync(rows.data(), h->series + R * first, sizeof(double) * R * count,
