@@ -60,6 +60,7 @@ __device__ __forceinline__ T lam_fold(const T *__restrict__ lam, long long plane
 // rows by two a thread, 4 CTAs of 256 threads with 64 registers (measured
 // fastest of 0, 3 and 4 CTAs, of one row a thread and of 2- and 8-row tiles:
 // 268 us a forward and backward step at 4096 x 2048 FP32 against 275-316).
+// FP64 takes half the CTAs (with 4 its 64 registers spilled 556 bytes).
 // Small grids, whose CTAs all fit the GPU at once, are one chain of latencies:
 // one row a thread in 2-row tiles, launched early (AdjSmall; 512 x 256 FP32:
 // 18.3 -> 15.3 us).
@@ -163,7 +164,11 @@ __device__ __forceinline__ typename Traits<S>::comp_t adj_node(const AdjArgs &a,
     const T jy = ((g[2] - g[4]) + (g[5] + g[6])) - (g[7] + g[8]);
     const T drho = (((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7]))) + g[8];
     const T rho = R0 + drho;
-    const T inv = T(1) / rho;
+    T inv;
+    if constexpr (sizeof(T) == 4)
+        inv = rcp_rn(rho);
+    else
+        inv = T(1) / rho;
     const T ux = jx * inv, uy = jy * inv;
     const T usq = ux * ux + uy * uy;
     const T om = param<T>(a.omega, a.omega_f);
@@ -224,7 +229,7 @@ __device__ __forceinline__ void adj_prefetch(const AdjArgs &a)
 }
 
 template <int S, typename G>
-__global__ void __launch_bounds__(adj_threads<G>(), G::MINB) k_adjoint_step(AdjArgs a)
+__global__ void __launch_bounds__(adj_threads<G>(), S == LBM_F64 ? G::MINB / 2 : G::MINB) k_adjoint_step(AdjArgs a)
 {
     constexpr int ADJ_TR = G::TR, ADJ_RPT = G::RPT, ADJ_WARPS = adj_warps<G>();
     using T = typename Traits<S>::comp_t;

@@ -1,6 +1,6 @@
-"""Multi-step passes (lbm_march.cu) against single steps: the staged kernel
-takes single steps on any grid, the direct kernel four at a time where the
-grid takes passes.  The populations and the link sums are the same bits, the
+"""Passes of four steps (lbm_march.cu; on small grids single-step launches with
+one link kernel) against single steps: the staged kernel takes single steps on
+any grid, the direct kernel four at a time where the grid takes passes.  The populations and the link sums are the same bits, the
 box sums too up to the order in which the staged kernel adds them."""
 import numpy as np
 import pytest
@@ -21,13 +21,13 @@ def gb():
 
 
 def body(name, nx, ny):
-    """none; a disc inside; a disc at the outlet; one that wraps through the top."""
+    """none; a disc inside; one at the inlet, one at the outlet; one that wraps through the top."""
     m = np.zeros((ny, nx), np.uint8)
     if name == "none":
         return m
     r = max(1.0, min(nx, ny) / 14)
     x, y = np.arange(nx)[None, :], np.arange(ny)[:, None]
-    cx, cy = {"disc": (0.4 * nx, 0.5 * ny), "outlet": (nx - 3 - r, 0.45 * ny), "wrap": (0.3 * nx, 0.0)}[name]
+    cx, cy = {"disc": (0.4 * nx, 0.5 * ny), "inlet": (2 + r, 0.55 * ny), "outlet": (nx - 3 - r, 0.45 * ny), "wrap": (0.3 * nx, 0.0)}[name]
     dy = np.abs(y - cy)
     m[(x - cx) ** 2 + np.minimum(dy, ny - dy) ** 2 <= r * r] = 1
     m[:, :2] = 0
@@ -42,10 +42,12 @@ def body(name, nx, ny):
 SIZES = [("f16dev", nx, ny) for nx, ny in
          [(16, 16), (64, 17), (119, 16), (120, 33), (121, 40), (122, 41), (123, 64), (240, 51), (241, 96), (500, 255)]]
 SIZES += [("f32dev", 1201, 751), ("f32", 1200, 751), ("f32dev", 1319, 700)]
+# small grids of the other storages: passes of single-step launches
+SIZES += [("f64", 131, 35), ("f32dev", 257, 66)]
 
 
 @pytest.mark.parametrize("storage,nx,ny", SIZES)
-@pytest.mark.parametrize("name", ["none", "disc", "outlet", "wrap"])
+@pytest.mark.parametrize("name", ["none", "disc", "inlet", "outlet", "wrap"])
 def test_passes_equal_single_steps(gb, storage, nx, ny, name):
     m = body(name, nx, ny)
     u = inputs.random_inlet(ny, seed=3, amp=0.002)
