@@ -46,6 +46,13 @@ constexpr int TIMING_BATCH = 64;
 // Multi-step passes per captured graph: long and short form (multiples of
 // NBUF, so that a graph ends on the buffer it starts from).
 constexpr int GRAPH_PASSES[2] = {12, NBUF};
+// Multi-step passes of grids from this many nodes on keep ahead of the GPU
+// when launched one by one (one takes 40 us and more, its launches 12-15 us of
+// the host's time), so a call of fewer than GRAPH_LONG_STEPS steps builds no
+// graph for them; a longer one replays the long form (1448 x 724: 10.2 against
+// 10.9 us a step; 4096 x 2048: 38.8 against 39.0).
+constexpr double GRAPH_NODES_MOST = 9e5;
+constexpr int GRAPH_LONG_STEPS = 192;
 // Share of the grid that the kept intermediate states may cover: with more of
 // it the pass writes so much that single steps are as fast.
 constexpr double MARCH_KEEP_SHARE = 0.25;
@@ -406,6 +413,7 @@ cudaError_t launch_link_side(lbm_ctx *h, int src, int precollision, int steps)
         pass_states(h, src, g.state, g.plane);
         g.steps = steps;
         for (int j = 0; j < steps; ++j) g.partials[j] = c.partials[j] = pass_partials(h, src, j);
+        g.early = h->pass_kind == PASS_STEPS;
         if (e == cudaSuccess) e = launch_cv_sums(h->storage, c, h->side, h->link_prio);
         h->launches += 1;
     }
@@ -634,6 +642,17 @@ void plan_passes(lbm_ctx *h, const std::vector<long long> &solids)
     if ((double)(k[1] - k[0] + 1) * (k[3] - k[2] + 1) > MARCH_KEEP_SHARE * h->nx * h->ny) return;
     memcpy(h->keep, k, sizeof(k));
     h->pass_kind = PASS_MARCH;
+}
+
+// Whether a pass is so short that the host's launches would hold it up.
+bool short_passes(const lbm_ctx *h) { return h->pass_kind != PASS_MARCH || (double)h->nx * h->ny < GRAPH_NODES_MOST; }
+
+// Whether the next passes of a call that has n steps to go come from a graph.
+bool replays(const lbm_ctx *h, int n)
+{
+    if (short_passes(h)) return n >= GRAPH_PASSES[1] * GROUP_STEPS;
+    return n >= GRAPH_PASSES[0] * GROUP_STEPS &&
+           (n >= GRAPH_LONG_STEPS || h->pass_graph[h->cur][0][0] || h->pass_graph[h->cur][0][1]);
 }
 
 // The buffers of the passes, at first use.  Without room for them
@@ -1052,7 +1071,7 @@ lbm_status queue_steps(lbm_ctx *h, int n)
             h->front_host = h->t;
             h->launches += 1;
         }
-        if (pass ? n < NBUF * GROUP_STEPS : (h->precollision || h->timing || n < NBUF || passes)) {
+        if (pass ? !replays(h, n) : (h->precollision || h->timing || n < NBUF || passes)) {
             cudaEvent_t *ev = h->timing ? &h->events[3 * nev] : nullptr;
             CK(h, pass ? launch_one_pass(h, h->cur) : launch_one_step(h, h->cur, h->precollision, ev), "step launch");
             if (h->timing && ++nev == TIMING_BATCH) {
@@ -1111,6 +1130,7 @@ cudaError_t launch_kept_group(lbm_ctx *h, const void *const *state, int set)
     cudaError_t e = h->ev_live[set] ? cudaStreamWaitEvent(h->stream, h->ev_read[set], 0) : cudaSuccess;
     LinkGroupArgs g = link_group(h, link_args(h, h->cur, next_buf(h->cur), 0, 0));
     g.steps = GROUP_STEPS;
+    g.early = 1;
     CvArgs c;
     memset(&c, 0, sizeof(c));
     c.s = step_args(h, h->cur, next_buf(h->cur), 0);
@@ -1345,7 +1365,7 @@ lbm_status lbm_prepare(lbm_ctx *h, long n)
     ensure_passes(h);
     const bool pass = h->pass_kind != PASS_NONE && !h->use_bulk;  // such a handle replays no graph of single steps
     for (int p = 0; p < NBUF; ++p)
-        for (int k = 0; k < 2; ++k)
+        for (int k = 0; k < (pass && !short_passes(h) ? 1 : 2); ++k)
             for (int l = 0; l < 2; ++l)
                 if (!(pass ? h->pass_graph : h->graph)[p][k][l]) {
                     st = build_graph(h, p, k, l, pass);

@@ -18,8 +18,8 @@
 //   link_partials [GROUP_STEPS][warps][14] per-warp rows of the link kernel, same types;
 //   series       double [steps][12]: A, B, DRTT, A', momentum defect, SI (x, y each);
 //   carry        double [8]: J_post(t-1), GL(t-1), flag;  step counter int64;
-//   ticket       uint32 arrival counters: of the link kernel's warps (one per
-//                step of a launch, one for the steps) and of the multi-step kernel.
+//   ticket       uint32 arrival counters of the link kernel's warps (one per
+//                step of a launch, one for the steps).
 #pragma once
 
 #include <cuda.h>
@@ -211,6 +211,7 @@ struct LinkArgs {
 struct LinkGroupArgs {
     LinkArgs a;
     int steps;
+    int early;               // launched while the box sums before it still run
     const void *state[GROUP_STEPS + 1];
     long long plane[GROUP_STEPS + 1];
     const double *partials[GROUP_STEPS];
