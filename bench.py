@@ -4,7 +4,9 @@
 One bench step is one lattice time step of the whole hot path: the fused
 collide-stream kernel over the grid (bounce-back, inlet/outlet, DRTT partials)
 plus the link kernel (momentum exchange A, A', B, DRTT and stress integration),
-forces of every scheme recorded on the device.  Default workload: 4096 x 2048 NACA0012, chord
+forces of every scheme recorded on the device.  Steps are taken four at a time
+(one pass of the multi-step kernel); the roofline entry is the single-step
+kernel's, timed launch by launch.  Default workload: 4096 x 2048 NACA0012, chord
 256 at 4 degrees, Re 1000, FP32 storage.  The population arrays (2 x 302 MB)
 exceed the 129 MB L2, so no flush is needed between steps.
 

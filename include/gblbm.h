@@ -146,16 +146,21 @@ void lbm_bc_default(lbm_bc *bc);
 lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const double *u_in,
                       int n_u_in, const lbm_bc *bc, lbm_ctx **out);
 
-/* Advance n >= 0 steps.  Each step t -> t+1 runs, in this order, the fused
- * pull-stream + bounce-back + inlet/outlet + BGK collision kernel (which also
- * accumulates J(t) and the control-volume fluxes), then the link kernel (MEA
- * A, A', B of step t and DRTT of step t-1).  Blocks until the work is done.
+/* Advance n >= 0 steps.  A step t -> t+1 is the fused pull-stream +
+ * bounce-back + inlet/outlet + BGK collision, J(t) and the control-volume
+ * fluxes, and the link sums (MEA A, A', B of step t and DRTT of step t-1).
+ * Four steps at a time are taken as one pass where the grid allows: by one
+ * kernel that takes every node four steps further (channels of FP32 and FP16
+ * storage, from a few hundred thousand nodes on, whose body and control volume
+ * cover a small part of the grid), or on small grids by four launches; either
+ * way with one link launch for the four.  Blocks until the work is done.
  * The call may be split into any sequence of calls with the same total: the
  * state and the force series do not depend on the split.
  * EUNSTABLE if any step produced rho <= 0 or NaN (the state then holds the
- * result after all n steps); ETIMEOUT if a bounded wait of the staged kernel
- * expired; ESTATE if a series row would have fallen outside the series buffer
- * (an internal invariant; the row is dropped rather than written). */
+ * result after all n steps); ETIMEOUT if a bounded wait of the staged or the
+ * multi-step kernel expired; ESTATE if a series row would have fallen outside
+ * the series buffer (an internal invariant; the row is dropped rather than
+ * written). */
 lbm_status lbm_step(lbm_ctx *h, int n);
 
 /* lbm_step without the wait: queues n >= 0 steps on the handle's stream and
@@ -170,9 +175,10 @@ lbm_status lbm_step_async(lbm_ctx *h, int n);
 lbm_status lbm_sync(lbm_ctx *h);
 
 /* Optional: make the next n steps launch-only.  Grows the force series to
- * hold n more steps and builds the captured step graphs for every starting
- * buffer, so that a following lbm_step(m <= n) does no allocation, stream
- * capture or graph instantiation, only launches.  (lbm_step does the same work
+ * hold n more steps, allocates the buffers of the passes and builds the
+ * captured step graphs for every starting buffer, so that a following
+ * lbm_step(m <= n) does no allocation, stream capture or graph instantiation,
+ * only launches.  (lbm_step does the same work
  * lazily when it is not called.)  Blocks.  EINVAL for n < 0; ENOMEM, ECUDA. */
 lbm_status lbm_prepare(lbm_ctx *h, long n);
 
