@@ -38,7 +38,7 @@ def body(name, nx, ny):
 # strips of 120 columns (16: one partial strip; 121 and 241: the outlet column
 # alone in the last one; 119 .. 123: the outlet in the halo of the strip
 # before), odd columns and rows, pieces of an odd number of rows; FP32 grids
-# take passes from 900,000 nodes on
+# take passes of the multi-step kernel from 600,000 nodes on
 SIZES = [("f16dev", nx, ny) for nx, ny in
          [(16, 16), (64, 17), (119, 16), (120, 33), (121, 40), (122, 41), (123, 64), (240, 51), (241, 96), (500, 255)]]
 SIZES += [("f32dev", 1201, 751), ("f32", 1200, 751), ("f32dev", 1319, 700)]
