@@ -1,7 +1,7 @@
 // lbm_api.cu -- the C ABI declared in include/gblbm.h: argument checks, device
-// memory, set-up sequence, the step loop (CUDA graphs of whole step pairs) and
+// memory, set-up sequence, the step loop (CUDA graphs of steps and of passes) and
 // read-back.  All arithmetic of the method runs in the kernels of
-// lbm_setup.cu and lbm_step.cu.
+// lbm_setup.cu, lbm_step.cu, lbm_march.cu and lbm_link.cu.
 #include <climits>
 #include <cmath>
 #include <cstdarg>
@@ -46,13 +46,15 @@ constexpr int TIMING_BATCH = 64;
 // Multi-step passes per captured graph: long and short form (multiples of
 // NBUF, so that a graph ends on the buffer it starts from).
 constexpr int GRAPH_PASSES[2] = {12, NBUF};
-// Multi-step passes of grids from this many nodes on keep ahead of the GPU
-// when launched one by one (one takes 40 us and more, its launches 12-15 us of
-// the host's time), so a call of fewer than GRAPH_LONG_STEPS steps builds no
-// graph for them; a longer one replays the long form (1448 x 724: 10.2 against
-// 10.9 us a step; 4096 x 2048: 38.8 against 39.0).
+// A call of fewer than GRAPH_LONG_STEPS steps builds no long form (a handle's
+// first call, 603 x 300 FP32: 100 steps 901 us with the long form, 809 with the
+// short one; 250 steps 1922 and 1884; 400 steps 2903 and 2943).  Multi-step
+// passes of grids from GRAPH_NODES_MOST nodes on keep ahead of the GPU when
+// launched one by one (one takes 40 us and more, its launches 12-15 us of the
+// host's time): such a call builds no graph for them; a longer one replays the
+// long form (1448 x 724: 10.2 against 10.9 us a step; 4096 x 2048: 38.8 against 39.0).
 constexpr double GRAPH_NODES_MOST = 9e5;
-constexpr int GRAPH_LONG_STEPS = 192;
+constexpr int GRAPH_LONG_STEPS = 384;
 // Share of the grid that the kept intermediate states may cover: with more of
 // it the pass writes so much that single steps are as fast.
 constexpr double MARCH_KEEP_SHARE = 0.25;
@@ -647,12 +649,17 @@ void plan_passes(lbm_ctx *h, const std::vector<long long> &solids)
 // Whether a pass is so short that the host's launches would hold it up.
 bool short_passes(const lbm_ctx *h) { return h->pass_kind != PASS_MARCH || (double)h->nx * h->ny < GRAPH_NODES_MOST; }
 
-// Whether the next passes of a call that has n steps to go come from a graph.
-bool replays(const lbm_ctx *h, int n)
+// Whether the next passes of a call that has n steps to go come from a long graph.
+bool long_form(const lbm_ctx *h, int n)
 {
-    if (short_passes(h)) return n >= GRAPH_PASSES[1] * GROUP_STEPS;
     return n >= GRAPH_PASSES[0] * GROUP_STEPS &&
            (n >= GRAPH_LONG_STEPS || h->pass_graph[h->cur][0][0] || h->pass_graph[h->cur][0][1]);
+}
+
+// Whether they come from a graph at all.
+bool replays(const lbm_ctx *h, int n)
+{
+    return short_passes(h) ? n >= GRAPH_PASSES[1] * GROUP_STEPS : long_form(h, n);
 }
 
 // The buffers of the passes, at first use.  Without room for them
@@ -1086,7 +1093,7 @@ lbm_status queue_steps(lbm_ctx *h, int n)
             if (pass) h->front_host += GROUP_STEPS;
         } else {
             const int each = pass ? GROUP_STEPS : 1;
-            const int k = n >= each * (pass ? GRAPH_PASSES[0] : GRAPH_STEPS) ? 0 : 1;
+            const int k = (pass ? long_form(h, n) : n >= GRAPH_STEPS) ? 0 : 1;
             const int units = pass ? GRAPH_PASSES[k] : (k == 0 ? GRAPH_STEPS : NBUF);
             // a held link kernel of the step or pass before opens the graph
             const int lead = h->lead_src == prev_buf(h->cur) && !h->lead_pre && h->lead_steps == each ? 1 : 0;
