@@ -1183,8 +1183,8 @@ lbm_status queue_steps_keep(lbm_ctx *h, int n, char *slots, size_t stride)
     lbm_status st = ensure_series(h, h->t + n);
     if (st == LBM_OK) st = arm_status(h);
     if (st != LBM_OK) return st;
-    if (n > GROUP_STEPS) ensure_passes(h);
-    const bool groups = h->pass_kind == PASS_STEPS;
+    if (n >= GROUP_STEPS) ensure_passes(h);
+    const bool groups = h->pass_kind == PASS_STEPS && h->group_partials;
     void *orig[NBUF];
     for (int b = 0; b < NBUF; ++b) orig[b] = h->pop[b];
     const int bulk = h->use_bulk, end = (h->cur + n) % NBUF;  // the buffer of the last state
