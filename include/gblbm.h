@@ -288,11 +288,11 @@ long lbm_num_links(const lbm_ctx *h);
  * same arithmetic per node.  Waits for the handle's stream. */
 lbm_status lbm_set_kernel(lbm_ctx *h, int kernel);
 
-/* Bound, in polls, on each pipeline wait of the staged kernel (default
- * 2^22; polls < 0 restores it).  For testing the timeout path: with 0, every
- * CTA's first wait gives up at once, the CTA waits (with a bound of its own)
- * for the copies it has issued, and lbm_step returns ETIMEOUT; the step's
- * output is then incomplete, and the caller restores a state
+/* Bound, in polls, on each pipeline wait of the staged and of the multi-step
+ * kernel (default 2^22; polls < 0 restores it).  For testing the timeout path:
+ * with 0, every CTA's first wait gives up at once, the CTA waits (with a bound
+ * of its own) for the copies it has issued, and lbm_step returns ETIMEOUT; the
+ * steps' output is then incomplete, and the caller restores a state
  * (lbm_set_populations) before stepping on.  Waits for the handle's stream. */
 lbm_status lbm_set_wait_limit(lbm_ctx *h, long polls);
 

@@ -318,7 +318,7 @@ class Lattice:
         _check(lib().lbm_set_kernel(self._h, {"direct": 0, "staged": 1}.get(kernel, kernel)), self._h)
 
     def set_wait_limit(self, polls):
-        """Poll bound of the staged kernel's pipeline waits (lbm_set_wait_limit;
+        """Poll bound of the staged and multi-step kernels' pipeline waits (lbm_set_wait_limit;
         negative: the default).  Only for testing the timeout path."""
         _check(lib().lbm_set_wait_limit(self._h, int(polls)), self._h)
 

@@ -96,7 +96,7 @@ struct lbm_ctx {
     int use_bulk = 0, sm_count = 1;
     int pf_rows = 0;                                     // L2 prefetch distance of the direct kernel
     int first_r0 = 1, first_r1 = 0;                      // tile rows holding bounce-back tiles (none: r0 > r1)
-    unsigned int wait_limit = WAIT_LIMIT;                // polls of each staged-kernel pipeline wait
+    unsigned int wait_limit = WAIT_LIMIT;                // polls of each pipeline wait of the staged and the multi-step kernel
     int cur = 0;                 // buffer holding the latest state
     cudaStream_t side = nullptr; // link kernels
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_read[NBUF] = {nullptr, nullptr, nullptr};

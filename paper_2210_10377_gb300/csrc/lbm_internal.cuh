@@ -161,7 +161,7 @@ struct StepArgs {
     int sm_count;            // persistent grid size of the staged kernel
     int pf_rows;             // L2 prefetch distance of the direct kernel in tile rows (0: off)
     int first_r0, first_r1;  // tile rows with bounce-back tiles, dispatched first (r0 > r1: none)
-    unsigned int wait_limit; // polls of each pipeline wait of the staged kernel (WAIT_LIMIT)
+    unsigned int wait_limit; // polls of each pipeline wait of the staged and the multi-step kernel
     int step_off;            // this launch's step is *step_ctr + step_off
     int pass;                // a step of a pass (step_off, early, next_ctr may be set)
     int early;               // launched while its predecessor may still run (see launch_collide_stream)
