@@ -142,6 +142,7 @@ struct lbm_ctx {
     long long series_cap = 0;
     double *carry = nullptr;     // [8]
     long long *step_ctr = nullptr;
+    long long *zero_ctr = nullptr;  // a word that stays 0: the counter of launches that carry their step number
     int *status = nullptr;       // [2]
     // Page-locked words that small results are read back into: settle's status
     // words, then one series row (a copy to pageable memory is staged, and the
@@ -451,12 +452,19 @@ cudaError_t join_side(lbm_ctx *h)
 // steps, not even across the end of a captured graph.  The collide-stream
 // kernel first waits for the link kernel of step t-2, which read the buffer
 // it overwrites.  With timing events (ev != NULL) both kernels run in order
-// on the handle's stream, each between events.
-cudaError_t launch_one_step(lbm_ctx *h, int src, int precollision, cudaEvent_t *ev)
+// on the handle's stream, each between events.  t: the step's number, for
+// reports, or -1 in a graph, whose launches read the step counter: it follows
+// the link kernels, which may lag the collide-stream kernels by a step, or by
+// the pass before.
+cudaError_t launch_one_step(lbm_ctx *h, int src, int precollision, cudaEvent_t *ev, long long t)
 {
     const int dst = next_buf(src);
     cudaError_t e = cudaSuccess;
     StepArgs sa = step_args(h, src, dst, precollision);
+    if (t >= 0) {
+        sa.step_ctr = h->zero_ctr;
+        sa.step_off = (int)t;
+    }
     if (ev) {
         if (h->lead_src >= 0) {
             e = flush_link(h);
@@ -558,7 +566,7 @@ lbm_status build_graph(lbm_ctx *h, int p, int k, int lead, bool passes)
     long long saved = h->launches;
     int b = p;
     for (int s = 0; s < units && le == cudaSuccess; ++s) {
-        le = passes ? launch_one_pass(h, b) : launch_one_step(h, b, 0, nullptr);
+        le = passes ? launch_one_pass(h, b) : launch_one_step(h, b, 0, nullptr, -1);
         b = next_buf(b);
     }
     if (le == cudaSuccess) le = join_side(h);
@@ -920,8 +928,9 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
     h->link_totals = h->link_partials + link_rows;
     ALLOC(h->ticket, unsigned int *, sizeof(unsigned int) * 16);
     ALLOC(h->carry, double *, sizeof(double) * 8);
-    ALLOC(h->step_ctr, long long *, sizeof(long long) * (1 + NBUF));
+    ALLOC(h->step_ctr, long long *, sizeof(long long) * (2 + NBUF));
     h->front = h->step_ctr + 1;
+    h->zero_ctr = h->front + NBUF;
     ALLOC(h->status, int *, sizeof(int) * 4);
     if (cudaHostAlloc((void **)&h->host_row, sizeof(double) * (2 + SERIES_ROW), cudaHostAllocDefault) != cudaSuccess) {
         cudaGetLastError();
@@ -939,7 +948,7 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
     CKC(cudaMemsetAsync(h->partials, 0, sizeof(double) * NBUF * CV_PARTIAL * h->n_cv_tiles, s), "memset");
     CKC(cudaMemsetAsync(h->ticket, 0, sizeof(unsigned int) * 16, s), "memset");
     CKC(cudaMemsetAsync(h->carry, 0, sizeof(double) * 8, s), "memset");
-    CKC(cudaMemsetAsync(h->step_ctr, 0, sizeof(long long) * (1 + NBUF), s), "memset");
+    CKC(cudaMemsetAsync(h->step_ctr, 0, sizeof(long long) * (2 + NBUF), s), "memset");
     const int status0[4] = {0, INT_MAX, 0, INT_MAX};  // the words, and what resets them
     CKC(cudaMemcpyAsync(h->status, status0, sizeof(status0), cudaMemcpyHostToDevice, s), "H2D status");
     h->status_armed = true;
@@ -1080,7 +1089,8 @@ lbm_status queue_steps(lbm_ctx *h, int n)
         }
         if (pass ? !replays(h, n) : (h->precollision || h->timing || n < NBUF || passes)) {
             cudaEvent_t *ev = h->timing ? &h->events[3 * nev] : nullptr;
-            CK(h, pass ? launch_one_pass(h, h->cur) : launch_one_step(h, h->cur, h->precollision, ev), "step launch");
+            CK(h, pass ? launch_one_pass(h, h->cur) : launch_one_step(h, h->cur, h->precollision, ev, h->t),
+               "step launch");
             if (h->timing && ++nev == TIMING_BATCH) {
                 st = flush_timing(h, nev);
                 if (st != LBM_OK) return st;
@@ -1217,7 +1227,7 @@ lbm_status queue_steps_keep(lbm_ctx *h, int n, char *slots, size_t stride)
         // the held link kernel of step j-1 reads buffers prev(cur) and cur,
         // whose addresses stay as they were
         h->pop[db] = state(j + 1);
-        e = launch_one_step(h, h->cur, h->precollision, nullptr);
+        e = launch_one_step(h, h->cur, h->precollision, nullptr, h->t);
         h->cur = db;
         h->precollision = 0;
         h->t += 1;
