@@ -144,10 +144,6 @@ struct lbm_ctx {
     long long *step_ctr = nullptr;
     long long *zero_ctr = nullptr;  // a word that stays 0: the counter of launches that carry their step number
     int *status = nullptr;       // [2]
-    // Page-locked words that small results are read back into: settle's status
-    // words, then one series row (a copy to pageable memory is staged, and the
-    // host waits for the staging).
-    double *host_row = nullptr;
     bool status_armed = false;   // status cleared for the queued steps
     bool pending = false;        // steps queued and not yet settled
     long long t = 0;
@@ -756,7 +752,6 @@ void free_all(lbm_ctx *h)
                     h->u_row, h->inlet, h->partials, h->link_partials, h->ticket, h->series,
                     h->carry, h->step_ctr, h->status, h->mid, h->group_partials, h->march_units_d};
     for (void *p : bufs) dev_free(h, p);
-    if (h->host_row) cudaFreeHost(h->host_row);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
 
@@ -932,10 +927,6 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
     h->front = h->step_ctr + 1;
     h->zero_ctr = h->front + NBUF;
     ALLOC(h->status, int *, sizeof(int) * 4);
-    if (cudaHostAlloc((void **)&h->host_row, sizeof(double) * (2 + SERIES_ROW), cudaHostAllocDefault) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(set_err(h, LBM_ENOMEM, "allocation of page-locked memory failed"));
-    }
     st = ensure_series(h, 1024);
     if (st != LBM_OK) return fail(st);
 
@@ -1037,7 +1028,7 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
 namespace {
 
 // Clears the status words for the steps about to be queued, unless the last
-// settle already did: status[0] = 0 (no flag), status[1] = INT_MAX (no bad
+// settle found them so: status[0] = 0 (no flag), status[1] = INT_MAX (no bad
 // step yet).
 lbm_status arm_status(lbm_ctx *h)
 {
@@ -1249,13 +1240,10 @@ lbm_status settle(lbm_ctx *h)
     if (!h->pending) return LBM_OK;
     h->pending = false;
     h->status_armed = false;
-    CK(h, cudaMemcpyAsync(h->host_row, h->status, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream), "D2H status");
-    // clear the words for the next queue here, so that its start waits on nothing
-    CK(h, cudaMemcpyAsync(h->status, h->status + 2, 2 * sizeof(int), cudaMemcpyDeviceToDevice, h->stream),
-       "status reset");
+    int status[2] = {0, 0};
+    CK(h, cudaMemcpyAsync(status, h->status, sizeof(status), cudaMemcpyDeviceToHost, h->stream), "D2H status");
     CK(h, cudaStreamSynchronize(h->stream), "step sync");
-    h->status_armed = true;
-    const int status[2] = {((const int *)h->host_row)[0], ((const int *)h->host_row)[1]};
+    h->status_armed = status[0] == 0;  // words that nothing raised are still cleared
     if (h->t - 1 > h->carry_from) h->drtt_ready = h->t - 1 > h->drtt_ready ? h->t - 1 : h->drtt_ready;
     if (status[0] & 4)
         return set_err(h, LBM_ESTATE, "a force-series row lay beyond the series buffer");
@@ -1315,7 +1303,7 @@ lbm_status lbm_force_series(lbm_ctx *h, int scheme, long first, long count, doub
     }
     const size_t R = SERIES_ROW;
     if (count == 1) {
-        double *row = h->host_row + 2;
+        double row[SERIES_ROW];
         CK(h, cudaMemcpyAsync(row, h->series + R * (h->record_series ? first : (first & 1)), sizeof(double) * R,
                               cudaMemcpyDeviceToHost, h->stream),
            "D2H series");

@@ -60,3 +60,22 @@ def test_first_unstable_step_does_not_depend_on_the_split(gb, storage):
             lat.step(1)
         assert reported(gb, lat, 2 * first) == first
         lat.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16dev"])
+def test_a_report_is_given_once_and_the_next_one_is_its_own(gb, storage):
+    # the status words are cleared after a report, and only then
+    nx, ny = 200, 64
+    lat = gb.Lattice(np.zeros((ny, nx), np.uint8), 0.5001, 0.1, storage=storage)
+    calm = lat.populations()
+    wild = inputs.random_populations(nx, ny, seed=8, lo=0.08, hi=0.14)
+    reports = []
+    for _ in range(2):
+        lat.set_populations(wild)
+        t0 = lat.steps_done
+        reports.append(reported(gb, lat, 399) - t0)
+        lat.set_populations(calm)
+        for n in (1, 9, 1):
+            lat.step(n)
+    assert reports[0] == reports[1]
+    lat.close()
