@@ -666,6 +666,18 @@ bool replays(const lbm_ctx *h, int n)
     return short_passes(h) ? n >= GRAPH_PASSES[1] * GROUP_STEPS : long_form(h, n);
 }
 
+// The control-volume rows of groups of steps, at first use (false: no room).
+bool ensure_group_rows(lbm_ctx *h)
+{
+    if (!h->group_partials)
+        h->group_partials =
+            (double *)dev_alloc(h, sizeof(double) * NBUF * GROUP_STEPS * CV_PARTIAL * h->n_cv_tiles);
+    return h->group_partials != nullptr;
+}
+
+// Whether the steps of a call run in passes where the grid takes them.
+bool takes_passes(const lbm_ctx *h) { return h->pass_kind != PASS_NONE && !h->use_bulk && !h->timing; }
+
 // The buffers of the passes, at first use.  Without room for them
 // the handle takes single steps.
 void ensure_passes(lbm_ctx *h)
@@ -673,9 +685,8 @@ void ensure_passes(lbm_ctx *h)
     if (h->pass_kind == PASS_NONE || h->mid) return;
     const size_t state = 9 * (size_t)mid_plane(h) * h->elem;
     h->mid = (char *)dev_alloc(h, state * NBUF * (GROUP_STEPS - 1));
-    h->group_partials = (double *)dev_alloc(h, sizeof(double) * NBUF * GROUP_STEPS * CV_PARTIAL * h->n_cv_tiles);
     // the kernels' copies and prefetches of rows start on 16-byte boundaries
-    bool ok = h->mid && h->group_partials && ((uintptr_t)h->mid & 15) == 0;
+    bool ok = h->mid && ((uintptr_t)h->mid & 15) == 0 && ensure_group_rows(h);
     if (ok && h->pass_kind == PASS_MARCH) {
         std::vector<int2> units;
         h->plan = march_plan(h->storage, h->nx, h->ny, h->sm_count, h->bounce, h->keep, &units);
@@ -1069,9 +1080,9 @@ lbm_status queue_steps(lbm_ctx *h, int n)
         return LBM_OK;
     }
     int nev = 0;
-    if (n >= GROUP_STEPS) ensure_passes(h);
+    if (takes_passes(h) && n - (h->precollision ? 1 : 0) >= GROUP_STEPS) ensure_passes(h);
     while (n > 0) {
-        const bool passes = h->pass_kind != PASS_NONE && !h->use_bulk && !h->timing;
+        const bool passes = takes_passes(h);
         const bool pass = passes && !h->precollision && n >= GROUP_STEPS;
         if (pass && h->front_host != h->t) {
             CK(h, launch_set_counter(h->front + h->cur, h->t, h->stream), "step counter");
@@ -1184,8 +1195,8 @@ lbm_status queue_steps_keep(lbm_ctx *h, int n, char *slots, size_t stride)
     lbm_status st = ensure_series(h, h->t + n);
     if (st == LBM_OK) st = arm_status(h);
     if (st != LBM_OK) return st;
-    if (n >= GROUP_STEPS) ensure_passes(h);
-    const bool groups = h->pass_kind == PASS_STEPS && h->group_partials;
+    const bool groups =
+        h->pass_kind == PASS_STEPS && n - (h->precollision ? 1 : 0) >= GROUP_STEPS && ensure_group_rows(h);
     void *orig[NBUF];
     for (int b = 0; b < NBUF; ++b) orig[b] = h->pop[b];
     const int bulk = h->use_bulk, end = (h->cur + n) % NBUF;  // the buffer of the last state
@@ -1367,8 +1378,8 @@ lbm_status lbm_prepare(lbm_ctx *h, long n)
     if (n < 0) return set_err(h, LBM_EINVAL, "n must be >= 0");
     lbm_status st = ensure_series(h, h->t + n);
     if (st != LBM_OK) return st;
-    ensure_passes(h);
-    const bool pass = h->pass_kind != PASS_NONE && !h->use_bulk;  // such a handle replays no graph of single steps
+    if (takes_passes(h)) ensure_passes(h);
+    const bool pass = takes_passes(h);  // such a handle replays no graph of single steps
     for (int p = 0; p < NBUF; ++p)
         for (int k = 0; k < (pass && !short_passes(h) ? 1 : 2); ++k)
             for (int l = 0; l < 2; ++l)
