@@ -1442,14 +1442,20 @@ lbm_status lbm_populations(lbm_ctx *h, double *out)
     const size_t N = (size_t)h->nx * h->ny;
     // Two scratch planes: while one plane is copied to the host on the side
     // stream, the next one is gathered on the handle's.  Small planes are
-    // gathered together and copied at once.
-    const bool together = 9 * sizeof(double) * N <= READ_TOGETHER_BYTES;
-    double *scratch = (double *)dev_alloc(h, sizeof(double) * N * (together ? 9 : 2));
+    // gathered together and copied at once.  One plane, gathered and copied in
+    // turn, where there is no room for more.
+    int planes = 9 * sizeof(double) * N <= READ_TOGETHER_BYTES ? 9 : 2;
+    double *scratch = (double *)dev_alloc(h, sizeof(double) * N * planes);
+    if (!scratch) {
+        planes = 1;
+        scratch = (double *)dev_alloc(h, sizeof(double) * N);
+    }
     if (!scratch) return set_err(h, LBM_ENOMEM, "scratch allocation failed");
+    const bool together = planes == 9;
     cudaError_t e = cudaSuccess;
     for (int i = 0; i < 9 && e == cudaSuccess; ++i) {
-        double *plane = scratch + (together ? i : i & 1) * N;
-        if (!together && i >= 2) e = cudaStreamWaitEvent(h->stream, h->ev_read[i & 1], 0);
+        double *plane = scratch + (i % planes) * N;
+        if (!together && i >= planes) e = cudaStreamWaitEvent(h->stream, h->ev_read[i % planes], 0);
         if (e == cudaSuccess)
             e = launch_gather(h->storage, h->pop[h->cur], h->nbits, h->inlet, h->plane, h->nx, h->ny, h->pitch,
                               h->periodic, h->precollision, h->rho0, i, plane, h->stream);
@@ -1459,7 +1465,7 @@ lbm_status lbm_populations(lbm_ctx *h, double *out)
         if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->ev_fork, 0);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(out + i * N, plane, sizeof(double) * N, cudaMemcpyDeviceToHost, h->side);
-        if (e == cudaSuccess) e = cudaEventRecord(h->ev_read[i & 1], h->side);
+        if (e == cudaSuccess) e = cudaEventRecord(h->ev_read[i % planes], h->side);
     }
     if (e == cudaSuccess && together)
         e = cudaMemcpyAsync(out, scratch, sizeof(double) * 9 * N, cudaMemcpyDeviceToHost, h->stream);

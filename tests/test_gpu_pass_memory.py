@@ -60,3 +60,50 @@ def test_kept_steps_of_a_gradient_take_no_states_of_passes(gb, storage):
     lat.adjoint(12, 5, 0.3, 0.7)
     assert held(lat) - before < state(storage)
     lat.close()
+
+
+@pytest.fixture
+def refusing(gb, monkeypatch):
+    """An allocator whose user can set the largest block that it hands out."""
+    limit = [None]
+    alloc = gb._TorchAllocator._alloc
+
+    def limited(self, nbytes, stream, user):
+        return None if limit[0] is not None and nbytes > limit[0] else alloc(self, nbytes, stream, user)
+
+    monkeypatch.setattr(gb._TorchAllocator, "_alloc", limited)
+    return limit
+
+
+@pytest.mark.parametrize("storage", ["f64", "f16dev"])
+def test_populations_need_room_for_one_plane_only(gb, refusing, storage):
+    lat = lattice(gb, storage)
+    lat.step(5)
+    want = lat.populations()
+    refusing[0] = 8 * NX * NY + 255  # one FP64 plane, rounded up to 256 bytes
+    assert np.array_equal(lat.populations(), want)
+    refusing[0] = 8 * NX * NY - 1
+    with pytest.raises(gb.LbmError) as e:
+        lat.populations()
+    assert e.value.code == 2
+    lat.close()
+
+
+@pytest.mark.parametrize("storage", ["f64", "f32dev", "f16dev"])
+def test_without_room_for_passes_steps_run_one_by_one(gb, refusing, storage):
+    runs = []
+    for refuse in (False, True):
+        refusing[0] = None
+        lat = lattice(gb, storage)
+        if refuse:
+            before = held(lat)
+            refusing[0] = 1024  # neither the states nor the rows of the passes
+        for n in (1, 30, 7):
+            lat.step(n)
+        if refuse:
+            assert held(lat) == before
+        refusing[0] = None
+        runs.append((lat.populations(), np.stack(lat.force_series("B")), np.stack(lat.force_series("DRTT"))))
+        lat.close()
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
