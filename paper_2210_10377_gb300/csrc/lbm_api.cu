@@ -211,22 +211,21 @@ void dev_free(lbm_ctx *h, void *p)
         cudaFree(p);
 }
 
-// cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda link).
+// cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda
+// link), looked up once; threads that create their first handles together wait
+// for the one that looks it up.
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
 {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    static const PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
         void *p = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
                 cudaSuccess &&
             q == cudaDriverEntryPointSuccess)
-            fn = (PFN_cuTensorMapEncodeTiled_v12000)p;
-        else
-            cudaGetLastError();
-    }
+            return (PFN_cuTensorMapEncodeTiled_v12000)p;
+        cudaGetLastError();
+        return nullptr;
+    }();
     return fn;
 }
 
