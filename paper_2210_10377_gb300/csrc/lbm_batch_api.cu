@@ -376,7 +376,21 @@ lbm_status ensure_passes(lbm_batch *b)
     if (e != cudaSuccess || !b->mid || ((uintptr_t)b->mid & 15) || !b->pass_partials || !b->pass_largs || !b->totals ||
         !b->tickets || !b->front) {
         cudaGetLastError();
-        b->pass_ok = false;  // what was handed out is given back with the batch
+        b->pass_ok = false;
+        void *got[] = {b->mid, b->pass_partials, b->pass_largs, b->totals, b->tickets, b->front};
+        for (void *p : got) bdev_free(b, p);
+        b->mid = nullptr;
+        b->pass_partials = nullptr;
+        b->pass_largs = nullptr;
+        b->totals = nullptr;
+        b->tickets = nullptr;
+        b->front = nullptr;
+        for (cudaEvent_t *ev : {&b->ev_fork, &b->ev_join, &b->ev_read}) {
+            if (*ev) cudaEventDestroy(*ev);
+            *ev = nullptr;
+        }
+        if (b->side) cudaStreamDestroy(b->side);
+        b->side = nullptr;
         return LBM_OK;
     }
     std::vector<LinkArgs> la(BATCH_SHAPES * slices * n);

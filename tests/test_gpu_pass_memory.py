@@ -107,3 +107,25 @@ def test_without_room_for_passes_steps_run_one_by_one(gb, refusing, storage):
         lat.close()
     for a, b in zip(*runs):
         assert np.array_equal(a, b)
+
+
+def test_a_batch_without_room_for_passes_gives_back_what_it_got(gb, refusing):
+    m = np.zeros((NY, NX), np.uint8)
+    m[28:36, 90:110] = 1
+    domains = [dict(mask=m, tau=0.6, u_in=0.05), dict(mask=np.zeros((40, 100), np.uint8), tau=0.7, u_in=0.03)]
+    runs = []
+    for refuse in (False, True):
+        refusing[0] = None
+        b = gb.Batch(domains, storage="f32")
+        if refuse:
+            before = held(b)
+            refusing[0] = state("f32")  # the tables of the passes, not their states
+        for n in (1, 30, 7):
+            b.step(n)
+        if refuse:
+            assert held(b) == before
+        refusing[0] = None
+        runs.append([b.populations(0), b.populations(1), *b.force_series(0, "B"), *b.force_series(0, "DRTT")])
+        b.close()
+    for x, y in zip(*runs):
+        assert np.array_equal(x, y)
