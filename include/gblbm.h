@@ -175,11 +175,13 @@ lbm_status lbm_step_async(lbm_ctx *h, int n);
 lbm_status lbm_sync(lbm_ctx *h);
 
 /* Optional: make the next n steps launch-only.  Grows the force series to
- * hold n more steps, allocates the buffers of the passes and builds the
- * captured step graphs for every starting buffer, so that a following
- * lbm_step(m <= n) does no allocation, stream capture or graph instantiation,
- * only launches.  (lbm_step does the same work
- * lazily when it is not called.)  Blocks.  EINVAL for n < 0; ENOMEM, ECUDA. */
+ * hold n more steps, allocates the buffers of the passes (n >= 4) and builds
+ * the captured graphs that a call of n steps or fewer replays, for every
+ * starting buffer, so that a following lbm_step(m <= n) does no allocation,
+ * stream capture or graph instantiation, only launches.  (lbm_step does the
+ * same work lazily when it is not called.)  The cost grows with n: on small
+ * grids about 60 us below 12 steps, 300 us up to 384 and 780 us above.  Blocks.
+ * EINVAL for n < 0; ENOMEM, ECUDA. */
 lbm_status lbm_prepare(lbm_ctx *h, long n);
 
 /* Force on the body (+x downstream) of the last completed step t = T-1

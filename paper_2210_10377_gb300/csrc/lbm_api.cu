@@ -43,9 +43,11 @@ constexpr double ADJ_KEEP_SHARE = GBLBM_ADJ_KEEP_SHARE;
 #define GBLBM_BODY_ROWS_FIRST 1
 #endif
 constexpr int TIMING_BATCH = 64;
-// Multi-step passes per captured graph: long and short form (multiples of
-// NBUF, so that a graph ends on the buffer it starts from).
-constexpr int GRAPH_PASSES[2] = {12, NBUF};
+// Graphs of passes (multiples of NBUF, so that a graph ends on the buffer it
+// starts from): the long and the short one, which open with the held link
+// kernel of the pass before, and the short one that begins a call.
+enum PassForm { FORM_LONG = 0, FORM_SHORT, FORM_FIRST, PASS_FORMS, FORM_NONE = -1 };
+constexpr int GRAPH_PASSES[PASS_FORMS] = {12, NBUF, NBUF};
 // A call of fewer than GRAPH_LONG_STEPS steps builds no long form (a handle's
 // first call, 603 x 300 FP32: 100 steps 901 us with the long form, 809 with the
 // short one; 250 steps 1922 and 1884; 400 steps 2903 and 2943).  Multi-step
@@ -152,8 +154,7 @@ struct lbm_ctx {
     long long drtt_ready = 0;    // DRTT(s) is final for s < drtt_ready
     // [start buffer][GRAPH_STEPS or NBUF steps][opens with the previous step's link kernel]
     cudaGraphExec_t graph[NBUF][2][2] = {};
-    // [start buffer][GRAPH_PASSES[k] passes][opens with the previous pass's link kernel]
-    cudaGraphExec_t pass_graph[NBUF][2][2] = {};
+    cudaGraphExec_t pass_graph[NBUF][PASS_FORMS] = {};  // [start buffer][form]
     bool timing = false;
     std::vector<cudaEvent_t> events;
     double kt_ms[2] = {0, 0};
@@ -534,16 +535,15 @@ void drop_graphs(lbm_ctx *h)
                     h->graph[p][k][l] = nullptr;
                 }
     for (int p = 0; p < NBUF; ++p)
-        for (int k = 0; k < 2; ++k)
-            for (int l = 0; l < 2; ++l)
-                if (h->pass_graph[p][k][l]) {
-                    cudaGraphExecDestroy(h->pass_graph[p][k][l]);
-                    h->pass_graph[p][k][l] = nullptr;
-                }
+        for (int k = 0; k < PASS_FORMS; ++k)
+            if (h->pass_graph[p][k]) {
+                cudaGraphExecDestroy(h->pass_graph[p][k]);
+                h->pass_graph[p][k] = nullptr;
+            }
 }
 
-// Captures GRAPH_STEPS (k = 0) or NBUF (k = 1) steps, or GRAPH_PASSES[k]
-// passes, from buffer p.  lead = 1: the graph opens with the held link kernel
+// Captures GRAPH_STEPS (k = 0) or NBUF (k = 1) steps, or the GRAPH_PASSES[k]
+// passes of form k, from buffer p.  lead = 1: the graph opens with the held link kernel
 // of the step or pass before (which read prev_buf(p)) beside its first
 // collide-stream kernel.  Either way the graph ends with its last link kernel
 // held: the caller sets lead_src.
@@ -575,7 +575,7 @@ lbm_status build_graph(lbm_ctx *h, int p, int k, int lead, bool passes)
         return cuda_err(h, le, "capture step kernels");
     }
     if (ee != cudaSuccess) return cuda_err(h, ee, "end capture");
-    cudaError_t ie = cudaGraphInstantiateWithFlags(passes ? &h->pass_graph[p][k][lead] : &h->graph[p][k][lead], g,
+    cudaError_t ie = cudaGraphInstantiateWithFlags(passes ? &h->pass_graph[p][k] : &h->graph[p][k][lead], g,
                                                    cudaGraphInstantiateFlagUseNodePriority);
     cudaGraphDestroy(g);
     if (ie != cudaSuccess) return cuda_err(h, ie, "instantiate graph");
@@ -652,17 +652,23 @@ void plan_passes(lbm_ctx *h, const std::vector<long long> &solids)
 // Whether a pass is so short that the host's launches would hold it up.
 bool short_passes(const lbm_ctx *h) { return h->pass_kind != PASS_MARCH || (double)h->nx * h->ny < GRAPH_NODES_MOST; }
 
-// Whether the next passes of a call that has n steps to go come from a long graph.
-bool long_form(const lbm_ctx *h, int n)
+// Whether the link kernel of the step or pass (of `steps`) before is held for
+// the next graph to open with.
+bool lead_held(const lbm_ctx *h, int steps)
 {
-    return n >= GRAPH_PASSES[0] * GROUP_STEPS &&
-           (n >= GRAPH_LONG_STEPS || h->pass_graph[h->cur][0][0] || h->pass_graph[h->cur][0][1]);
+    return h->lead_src == prev_buf(h->cur) && !h->lead_pre && h->lead_steps == steps;
 }
 
-// Whether they come from a graph at all.
-bool replays(const lbm_ctx *h, int n)
+// The graph from which the next passes of a call that has n steps to go come,
+// or FORM_NONE: they are launched one by one.
+int pass_form(const lbm_ctx *h, int n)
 {
-    return short_passes(h) ? n >= GRAPH_PASSES[1] * GROUP_STEPS : long_form(h, n);
+    if (lead_held(h, GROUP_STEPS)) {
+        if (n >= GRAPH_PASSES[FORM_LONG] * GROUP_STEPS && (n >= GRAPH_LONG_STEPS || h->pass_graph[h->cur][FORM_LONG]))
+            return FORM_LONG;
+        return short_passes(h) && n >= GRAPH_PASSES[FORM_SHORT] * GROUP_STEPS ? FORM_SHORT : FORM_NONE;
+    }
+    return short_passes(h) && n >= GRAPH_PASSES[FORM_FIRST] * GROUP_STEPS ? FORM_FIRST : FORM_NONE;
 }
 
 // The control-volume rows of groups of steps, at first use (false: no room).
@@ -1091,7 +1097,8 @@ lbm_status queue_steps(lbm_ctx *h, int n)
         // single steps behind others run directly (a graph would first wait for
         // the held link kernel); a call of just NBUF steps replays their graph
         // (512 x 256 FP32 deviations: 70 us directly, 61 us from the graph)
-        if (pass ? !replays(h, n) : (h->precollision || h->timing || n < NBUF || (passes && h->lead_src >= 0))) {
+        const int form = pass ? pass_form(h, n) : FORM_NONE;
+        if (pass ? form == FORM_NONE : (h->precollision || h->timing || n < NBUF || (passes && h->lead_src >= 0))) {
             cudaEvent_t *ev = h->timing ? &h->events[3 * nev] : nullptr;
             CK(h, pass ? launch_one_pass(h, h->cur) : launch_one_step(h, h->cur, h->precollision, ev, h->t),
                "step launch");
@@ -1107,14 +1114,14 @@ lbm_status queue_steps(lbm_ctx *h, int n)
             if (pass) h->front_host += GROUP_STEPS;
         } else {
             const int each = pass ? GROUP_STEPS : 1;
-            const int k = (pass ? long_form(h, n) : n >= GRAPH_STEPS) ? 0 : 1;
+            const int k = pass ? form : (n >= GRAPH_STEPS ? 0 : 1);
             const int units = pass ? GRAPH_PASSES[k] : (k == 0 ? GRAPH_STEPS : NBUF);
             // a held link kernel of the step or pass before opens the graph
-            const int lead = h->lead_src == prev_buf(h->cur) && !h->lead_pre && h->lead_steps == each ? 1 : 0;
+            const int lead = lead_held(h, each) ? 1 : 0;
             if (!lead) CK(h, flush_link(h), "link launch");
             // the graph's first steps overwrite buffers that launched link kernels read
             CK(h, join_side(h), "join");
-            cudaGraphExec_t *g = pass ? &h->pass_graph[h->cur][k][lead] : &h->graph[h->cur][k][lead];
+            cudaGraphExec_t *g = pass ? &h->pass_graph[h->cur][k] : &h->graph[h->cur][k][lead];
             if (!*g) {
                 st = build_graph(h, h->cur, k, lead, pass);
                 if (st != LBM_OK) return st;
@@ -1380,20 +1387,30 @@ lbm_status lbm_prepare(lbm_ctx *h, long n)
     if (n < 0) return set_err(h, LBM_EINVAL, "n must be >= 0");
     lbm_status st = ensure_series(h, h->t + n);
     if (st != LBM_OK) return st;
-    if (takes_passes(h)) ensure_passes(h);
-    const bool pass = takes_passes(h);  // such a handle replays the shortest graph of single steps only
-    for (int p = 0; pass && p < NBUF; ++p)
-        if (!h->graph[p][1][0]) {
-            st = build_graph(h, p, 1, 0, false);
-            if (st != LBM_OK) return st;
-        }
-    for (int p = 0; p < NBUF; ++p)
-        for (int k = 0; k < (pass && !short_passes(h) ? 1 : 2); ++k)
-            for (int l = 0; l < 2; ++l)
-                if (!(pass ? h->pass_graph : h->graph)[p][k][l]) {
-                    st = build_graph(h, p, k, l, pass);
-                    if (st != LBM_OK) return st;
-                }
+    // what a call of at most n steps can replay, from every starting buffer
+    if (takes_passes(h) && n >= GROUP_STEPS) ensure_passes(h);
+    const bool pass = takes_passes(h);
+    auto build = [&](bool passes, int k, int lead) {
+        for (int p = 0; p < NBUF; ++p)
+            if (!(passes ? h->pass_graph[p][k] : h->graph[p][k][lead])) {
+                const lbm_status r = build_graph(h, p, k, lead, passes);
+                if (r != LBM_OK) return r;
+            }
+        return LBM_OK;
+    };
+    if (n >= NBUF) st = build(false, 1, 0);
+    if (!pass) {
+        if (st == LBM_OK && n >= 2 * NBUF) st = build(false, 1, 1);
+        if (st == LBM_OK && n >= GRAPH_STEPS) st = build(false, 0, 0);
+        if (st == LBM_OK && n >= 2 * GRAPH_STEPS) st = build(false, 0, 1);
+    } else {
+        const int first = GRAPH_PASSES[FORM_FIRST] * GROUP_STEPS;  // steps before the others
+        if (st == LBM_OK && short_passes(h) && n >= first) st = build(true, FORM_FIRST, 0);
+        if (st == LBM_OK && short_passes(h) && n >= first + GRAPH_PASSES[FORM_SHORT] * GROUP_STEPS)
+            st = build(true, FORM_SHORT, 1);
+        if (st == LBM_OK && n > GRAPH_LONG_STEPS) st = build(true, FORM_LONG, 1);
+    }
+    if (st != LBM_OK) return st;
     return LBM_OK;
 }
 

@@ -41,8 +41,11 @@ namespace {
 #define GBLBM_BATCH_PATH_ORDER_F32 0
 #endif
 constexpr int BATCH_GRAPH_STEPS = 16;  // steps per captured graph (even: ends on the start buffer)
-// Passes per captured graph (even: ends on the start buffer).
-constexpr int BATCH_GRAPH_PASSES[2] = {8, 2};
+// Graphs of passes (an even number: they end on the start buffer): the long and
+// the short one, which open with the held link kernel of the pass before, and
+// the short one that begins a call.
+enum PassForm { FORM_LONG = 0, FORM_SHORT, FORM_FIRST, PASS_FORMS };
+constexpr int BATCH_GRAPH_PASSES[PASS_FORMS] = {8, 2, 2};
 // Batches up to this arena size take passes (six arenas more).  A link kernel
 // after every step, alone on the GPU for its 15-20 us, was half the step of
 // the cylinder study's batch (35 MB: 25 us a step) and a third of 12 airfoil
@@ -131,8 +134,7 @@ struct lbm_batch {
     bool read_live = false;       // a link kernel of a pass is on the side stream
     int held = -1;                // the pass whose link kernel is not queued yet (its source buffer)
     int link_prio = 0;
-    // [start buffer][BATCH_GRAPH_PASSES][opens with the previous pass's link kernel]
-    cudaGraphExec_t pass_graph[2][2][2] = {};
+    cudaGraphExec_t pass_graph[2][PASS_FORMS] = {};  // [start buffer][form]
     long long launches = 0;
     std::string err;
 };
@@ -197,12 +199,11 @@ void drop_graphs(lbm_batch *b)
                 b->graph[c][k] = nullptr;
             }
     for (int c = 0; c < 2; ++c)
-        for (int k = 0; k < 2; ++k)
-            for (int l = 0; l < 2; ++l)
-                if (b->pass_graph[c][k][l]) {
-                    cudaGraphExecDestroy(b->pass_graph[c][k][l]);
-                    b->pass_graph[c][k][l] = nullptr;
-                }
+        for (int k = 0; k < PASS_FORMS; ++k)
+            if (b->pass_graph[c][k]) {
+                cudaGraphExecDestroy(b->pass_graph[c][k]);
+                b->pass_graph[c][k] = nullptr;
+            }
 }
 
 void free_all(lbm_batch *b)
@@ -510,16 +511,16 @@ cudaError_t launch_pass(lbm_batch *b, int c)
     return e;
 }
 
-// Captures BATCH_GRAPH_STEPS (k = 0) or 2 steps, or BATCH_GRAPH_PASSES[k]
-// passes, from buffer c.  lead: the graph opens with the held link kernel of
-// the pass before.  A graph of passes ends with its last link kernel held.
-lbm_status build_graph(lbm_batch *b, int c, int k, bool passes, int lead)
+// Captures BATCH_GRAPH_STEPS (k = 0) or 2 steps, or the BATCH_GRAPH_PASSES[k]
+// passes of form k, from buffer c.  A graph of passes ends with its last link
+// kernel held.
+lbm_status build_graph(lbm_batch *b, int c, int k, bool passes)
 {
     const int units = passes ? BATCH_GRAPH_PASSES[k] : (k == 0 ? BATCH_GRAPH_STEPS : 2);
     cudaGraph_t g = nullptr;
     const long long saved = b->launches;
     const int saved_held = b->held;
-    if (passes) b->held = lead ? 1 - c : -1;
+    if (passes) b->held = k == FORM_FIRST ? -1 : 1 - c;
     b->read_live = false;
     BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
     cudaError_t le = cudaSuccess;
@@ -538,7 +539,7 @@ lbm_status build_graph(lbm_batch *b, int c, int k, bool passes, int lead)
         return bcuda(b, le, "capture batch steps");
     }
     if (ee != cudaSuccess) return bcuda(b, ee, "end capture");
-    cudaError_t ie = cudaGraphInstantiateWithFlags(passes ? &b->pass_graph[c][k][lead] : &b->graph[c][k], g,
+    cudaError_t ie = cudaGraphInstantiateWithFlags(passes ? &b->pass_graph[c][k] : &b->graph[c][k], g,
                                                    passes ? cudaGraphInstantiateFlagUseNodePriority : 0);
     cudaGraphDestroy(g);
     if (ie != cudaSuccess) return bcuda(b, ie, "instantiate graph");
@@ -930,25 +931,26 @@ lbm_status lbm_batch_step(lbm_batch *b, int n)
             b->front_host = b->t;
             b->launches += 1;
         }
-        if (pass && n < BATCH_GRAPH_PASSES[1] * GROUP_STEPS) {
+        if (pass && n < BATCH_GRAPH_PASSES[FORM_SHORT] * GROUP_STEPS) {
             BCK(b, launch_pass(b, b->cur), "batch pass launch");
             b->cur = 1 - b->cur;
             b->t += GROUP_STEPS;
             b->front_host = b->t;
             n -= GROUP_STEPS;
         } else if (pass) {
-            const int k = n >= BATCH_GRAPH_PASSES[0] * GROUP_STEPS ? 0 : 1;
-            const int lead = b->held >= 0 ? 1 : 0;
+            const int k = b->held < 0                                        ? FORM_FIRST
+                          : n >= BATCH_GRAPH_PASSES[FORM_LONG] * GROUP_STEPS ? FORM_LONG
+                                                                             : FORM_SHORT;
             // the graph's first pass overwrites buffers that launched link kernels read
             BCK(b, join_side(b), "join");
-            if (!b->pass_graph[b->cur][k][lead]) {
-                st = build_graph(b, b->cur, k, true, lead);
+            if (!b->pass_graph[b->cur][k]) {
+                st = build_graph(b, b->cur, k, true);
                 if (st != LBM_OK) return st;
             }
-            BCK(b, cudaGraphLaunch(b->pass_graph[b->cur][k][lead], b->stream), "graph launch");
+            BCK(b, cudaGraphLaunch(b->pass_graph[b->cur][k], b->stream), "graph launch");
             const int passes = BATCH_GRAPH_PASSES[k];
             b->held = 1 - b->cur;  // an even number of passes: the last one read the other buffer
-            b->launches += ((long long)n_chunks(b) * GROUP_STEPS + 1) * passes - (1 - lead);
+            b->launches += ((long long)n_chunks(b) * GROUP_STEPS + 1) * passes - (k == FORM_FIRST ? 1 : 0);
             b->t += (long long)passes * GROUP_STEPS;
             b->front_host = b->t;
             n -= passes * GROUP_STEPS;
@@ -965,7 +967,7 @@ lbm_status lbm_batch_step(lbm_batch *b, int n)
             const int k = n >= BATCH_GRAPH_STEPS ? 0 : 1;
             const int steps = k == 0 ? BATCH_GRAPH_STEPS : 2;
             if (!b->graph[b->cur][k]) {
-                st = build_graph(b, b->cur, k, false, 0);
+                st = build_graph(b, b->cur, k, false);
                 if (st != LBM_OK) return st;
             }
             BCK(b, cudaGraphLaunch(b->graph[b->cur][k], b->stream), "graph launch");
@@ -1074,21 +1076,23 @@ lbm_status lbm_batch_prepare(lbm_batch *b, long n)
     if (n < 0) return berr(b, LBM_EINVAL, "n must be >= 0");
     lbm_status st = ensure_series(b, b->t + n);
     if (st != LBM_OK) return st;
-    st = ensure_passes(b);
+    // what a call of at most n steps can replay, from either buffer
+    if (n >= GROUP_STEPS) st = ensure_passes(b);
+    auto build = [&](bool passes, int k) {
+        for (int c = 0; c < 2; ++c)
+            if (!(passes ? b->pass_graph[c][k] : b->graph[c][k])) {
+                const lbm_status r = build_graph(b, c, k, passes);
+                if (r != LBM_OK) return r;
+            }
+        return LBM_OK;
+    };
+    if (st == LBM_OK && n >= 2) st = build(false, 1);
+    if (st == LBM_OK && !b->pass_ok && n >= BATCH_GRAPH_STEPS) st = build(false, 0);
+    const int first = BATCH_GRAPH_PASSES[FORM_FIRST] * GROUP_STEPS;  // steps before the others
+    if (st == LBM_OK && b->pass_ok && n >= first) st = build(true, FORM_FIRST);
+    for (int k : {FORM_SHORT, FORM_LONG})
+        if (st == LBM_OK && b->pass_ok && n - first >= BATCH_GRAPH_PASSES[k] * GROUP_STEPS) st = build(true, k);
     if (st != LBM_OK) return st;
-    // a batch that takes passes replays the shortest graph of single steps only
-    for (int c = 0; b->pass_ok && c < 2; ++c)
-        if (!b->graph[c][1]) {
-            st = build_graph(b, c, 1, false, 0);
-            if (st != LBM_OK) return st;
-        }
-    for (int c = 0; c < 2; ++c)
-        for (int k = 0; k < 2; ++k)
-            for (int lead = 0; lead < (b->pass_ok ? 2 : 1); ++lead)
-                if (!(b->pass_ok ? b->pass_graph[c][k][lead] : b->graph[c][k])) {
-                    st = build_graph(b, c, k, b->pass_ok, lead);
-                    if (st != LBM_OK) return st;
-                }
     return LBM_OK;
 }
 

@@ -129,3 +129,25 @@ def test_a_batch_without_room_for_passes_gives_back_what_it_got(gb, refusing):
         b.close()
     for x, y in zip(*runs):
         assert np.array_equal(x, y)
+
+
+def test_preparing_fewer_steps_than_a_pass_takes_no_memory_for_passes(gb):
+    for storage in ("f64", "f16dev"):
+        lat = lattice(gb, storage)
+        before = held(lat)
+        lat.prepare(3)
+        assert held(lat) == before
+        lat.prepare(4)
+        taken = held(lat)
+        assert taken > before
+        lat.step(4)
+        lat.step(4)
+        assert held(lat) == taken
+        lat.close()
+    b = gb.Batch([dict(mask=np.zeros((40, 100), np.uint8), tau=0.7, u_in=0.03)], storage="f32")
+    before = held(b)
+    b.prepare(3)
+    assert held(b) == before
+    b.prepare(4)
+    assert held(b) > before
+    b.close()
