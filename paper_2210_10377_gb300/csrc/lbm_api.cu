@@ -111,6 +111,7 @@ struct lbm_ctx {
     // the multi-step kernel, and the intermediate states (of the rows `keep`),
     // one set per source buffer, allocated at first use.
     int pass_kind = PASS_NONE;
+    long long pass_asked = 0;     // steps of the calls so far that could have run in passes
     alignas(64) CUtensorMap pmap[NBUF];  // one-row boxes of the population buffers
     MarchPlan plan;
     int bounce[4] = {1, 0, 1, 0}, keep[4] = {1, 0, 1, 0};
@@ -683,6 +684,19 @@ bool ensure_group_rows(lbm_ctx *h)
 // Whether the steps of a call run in passes where the grid takes them.
 bool takes_passes(const lbm_ctx *h) { return h->pass_kind != PASS_NONE && !h->use_bulk && !h->timing; }
 
+// The steps that a handle's calls have to ask for before its passes are set up
+// (fewer run one by one, without building graphs that passes would not use).
+// The multi-step kernel's plan and buffers take 80-150 us, which four or five
+// passes give back; the buffers of single-step passes from a caching allocator
+// 10 us, which one pass does; cudaMalloc up to 150 us more.  First calls, before
+// passes -> set up at once -> by this rule: 12 steps at 1280 x 640 FP16 285 -> 330
+// -> 260 us, at 1500 x 125 FP32 with cudaMalloc 198 -> 290 -> 175; 20 steps 473 -> 450
+// -> 446 and 324 -> 383 -> 264.
+long long pass_setup_steps(const lbm_ctx *h)
+{
+    return (h->pass_kind == PASS_MARCH ? 20 : GROUP_STEPS) + (h->alloc_fn ? 0 : 32);
+}
+
 // The buffers of the passes, at first use.  Without room for them
 // the handle takes single steps.
 void ensure_passes(lbm_ctx *h)
@@ -1085,20 +1099,25 @@ lbm_status queue_steps(lbm_ctx *h, int n)
         return LBM_OK;
     }
     int nev = 0;
-    if (takes_passes(h) && n - (h->precollision ? 1 : 0) >= GROUP_STEPS) ensure_passes(h);
+    if (takes_passes(h) && n - (h->precollision ? 1 : 0) >= GROUP_STEPS) {
+        h->pass_asked += n;
+        if (h->pass_asked >= pass_setup_steps(h)) ensure_passes(h);
+    }
+    const bool passes = takes_passes(h);
     while (n > 0) {
-        const bool passes = takes_passes(h);
-        const bool pass = passes && !h->precollision && n >= GROUP_STEPS;
+        const bool pass = passes && h->mid && !h->precollision && n >= GROUP_STEPS;
         if (pass && h->front_host != h->t) {
             CK(h, launch_set_counter(h->front + h->cur, h->t, h->stream), "step counter");
             h->front_host = h->t;
             h->launches += 1;
         }
-        // single steps behind others run directly (a graph would first wait for
-        // the held link kernel); a call of just NBUF steps replays their graph
-        // (512 x 256 FP32 deviations: 70 us directly, 61 us from the graph)
+        // Where the grid takes passes, single steps run directly (behind others
+        // a graph would first wait for the held link kernel), but a call of just
+        // NBUF steps replays their graph (512 x 256 FP32 deviations: 70 us
+        // directly, 61 us from the graph).
         const int form = pass ? pass_form(h, n) : FORM_NONE;
-        if (pass ? form == FORM_NONE : (h->precollision || h->timing || n < NBUF || (passes && h->lead_src >= 0))) {
+        if (pass ? form == FORM_NONE
+                 : (h->precollision || h->timing || n < NBUF || (passes && (n > NBUF || h->lead_src >= 0)))) {
             cudaEvent_t *ev = h->timing ? &h->events[3 * nev] : nullptr;
             CK(h, pass ? launch_one_pass(h, h->cur) : launch_one_step(h, h->cur, h->precollision, ev, h->t),
                "step launch");

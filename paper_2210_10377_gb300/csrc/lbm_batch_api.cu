@@ -120,6 +120,7 @@ struct lbm_batch {
     cudaGraphExec_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
     // passes (allocated at first use; pass_ok: the batch takes them)
     bool pass_ok = false;
+    long long pass_asked = 0;     // steps of the calls so far that could have run in passes
     size_t arena_bytes = 0;       // one population arena with its guards
     long long part_rows = 0;      // rows of one partials slice
     char *mid = nullptr;          // [2][GROUP_STEPS - 1] arenas: the steps in between of the pass from each buffer
@@ -915,8 +916,13 @@ lbm_status lbm_batch_step(lbm_batch *b, int n)
     if (n == 0) return LBM_OK;
     lbm_status st = ensure_series(b, b->t + n);
     if (st != LBM_OK) return st;
-    if (n >= GROUP_STEPS) {
-        st = ensure_passes(b);
+    // The passes are set up once a batch's calls have asked for this many steps:
+    // it takes 40-100 us, with cudaMalloc 80 us more, and a pass gives back 20-30
+    // (first calls of 4, 8 and 20 steps, five cylinders, before passes -> set up at
+    // once -> by this rule: 164, 288, 744 -> 202, 305, 561 -> 159, 297, 565 us).
+    if (b->pass_ok && n - (b->t == 0 ? 1 : 0) >= GROUP_STEPS) {
+        b->pass_asked += n;
+        if (b->pass_asked >= (b->alloc_fn ? 20 : 32)) st = ensure_passes(b);
         if (st != LBM_OK) return st;
     }
     // In a batch that takes passes the single steps behind one (or behind the
@@ -925,7 +931,7 @@ lbm_status lbm_batch_step(lbm_batch *b, int n)
     // directly, 87 us from the graph).
     const bool direct = b->pass_ok && (b->t == 0 || n >= GROUP_STEPS);
     while (n > 0) {
-        const bool pass = b->pass_ok && b->t > 0 && n >= GROUP_STEPS;
+        const bool pass = b->pass_ok && b->mid && b->t > 0 && n >= GROUP_STEPS;
         if (pass && b->front_host != b->t) {
             BCK(b, launch_set_counter(b->front + b->cur, b->t, b->stream), "step counter");
             b->front_host = b->t;

@@ -30,7 +30,7 @@ def test_an_expired_wait_is_reported_and_the_handle_recovers(gb, storage, nx, ny
     m[ny // 2, nx // 3:nx // 3 + 3] = 1
     u = inputs.random_inlet(ny, seed=3, amp=0.002)
     lat = gb.Lattice(m, 0.56, u, storage=storage)
-    lat.step(9)
+    lat.step(33)
     f = lat.populations()
     lat.set_wait_limit(0)
     lat.step(3)  # single steps of the direct kernel wait on nothing

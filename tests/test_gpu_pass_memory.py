@@ -151,3 +151,18 @@ def test_preparing_fewer_steps_than_a_pass_takes_no_memory_for_passes(gb):
     b.prepare(4)
     assert held(b) > before
     b.close()
+
+
+@pytest.mark.parametrize("torch_alloc", [True, False])
+@pytest.mark.parametrize("storage", ["f64", "f32dev", "f16dev"])
+def test_calls_before_the_passes_are_set_up(gb, storage, torch_alloc):
+    # short calls run one by one until enough steps were asked for; the same bits
+    runs = []
+    for chunks in ([5, 3, 7, 4, 9, 12, 30, 2], [1] * 72):
+        lat = lattice(gb, storage, torch_alloc=torch_alloc)
+        for n in chunks:
+            lat.step(n)
+        runs.append([lat.populations()] + [np.stack(lat.force_series(s)) for s in ("A", "B", "SI", "DRTT")])
+        lat.close()
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
