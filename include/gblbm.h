@@ -154,6 +154,13 @@ lbm_status lbm_create(const uint8_t *mask, int nx, int ny, double tau, const dou
  * storage, from a few hundred thousand nodes on, whose body and control volume
  * cover a small part of the grid), or on small grids by four launches; either
  * way with one link launch for the four.  Blocks until the work is done.
+ * Passes hold device memory beside the handle's three states: nine states more
+ * on small grids (a state of 40 MB at most), nine times the full rows around
+ * body and control volume where the multi-step kernel runs (all rows if these
+ * reach the top or bottom edge).  It is taken once the handle's calls have
+ * asked for 4 to 52 steps that could run in passes, or by lbm_prepare; without
+ * room for it the steps run one by one.  Staged handles and handles with kernel
+ * timing on take none.
  * The call may be split into any sequence of calls with the same total: the
  * state and the force series do not depend on the split.
  * EUNSTABLE if any step produced rho <= 0 or NaN (the state then holds the
@@ -407,7 +414,10 @@ lbm_status lbm_batch_create(const lbm_domain *domains, int n, const lbm_bc *bc, 
  * Blocks until the work is done.  EUNSTABLE when any domain's instability
  * flag is set (the flags are sticky; lbm_batch_status names the domains);
  * every domain has still taken all n steps.  ESTATE if a series row would
- * have fallen outside the series buffer (an internal invariant). */
+ * have fallen outside the series buffer (an internal invariant).
+ * A batch whose states take 192 MB at most runs four steps at a time with one
+ * link launch for the four, and holds six states of the batch more beside its
+ * two (1.2 GB at most), taken and done without as lbm_step does. */
 lbm_status lbm_batch_step(lbm_batch *b, int n);
 
 /* Forces of every domain at one step (0 <= step < steps done), for a scheme
@@ -424,9 +434,11 @@ lbm_status lbm_batch_coefficients(lbm_batch *b, int domain, int scheme, long fir
                                   double u_ref, double *cd, double *cl, double *stats);
 
 /* Optional: make the next n batch steps launch-only (as lbm_prepare): grows
- * the series and builds the captured step graphs of both starting buffers for
+ * the series, allocates the buffers of the passes (n >= 4) and builds the graphs
+ * that a call of n steps or fewer replays, of both starting buffers, for
  * the current launch configuration (a later lbm_batch_set_launch or
- * lbm_batch_autotune that changes it drops them again). */
+ * lbm_batch_autotune that changes it drops them again).  About 200 us below 8
+ * steps, 740 us from 40 on. */
 lbm_status lbm_batch_prepare(lbm_batch *b, long n);
 
 /* Pre-collision populations of one domain at the current step: out is double

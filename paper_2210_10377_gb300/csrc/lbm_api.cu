@@ -49,12 +49,13 @@ constexpr int TIMING_BATCH = 64;
 enum PassForm { FORM_LONG = 0, FORM_SHORT, FORM_FIRST, PASS_FORMS, FORM_NONE = -1 };
 constexpr int GRAPH_PASSES[PASS_FORMS] = {12, NBUF, NBUF};
 // A call of fewer than GRAPH_LONG_STEPS steps builds no long form (a handle's
-// first call, 603 x 300 FP32: 100 steps 901 us with the long form, 809 with the
-// short one; 250 steps 1922 and 1884; 400 steps 2903 and 2943).  Multi-step
-// passes of grids from GRAPH_NODES_MOST nodes on keep ahead of the GPU when
-// launched one by one (one takes 40 us and more, its launches 12-15 us of the
-// host's time): such a call builds no graph for them; a longer one replays the
-// long form (1448 x 724: 10.2 against 10.9 us a step; 4096 x 2048: 38.8 against 39.0).
+// first call, 603 x 300 FP32: 100 steps 913 us with the long form, 807 without;
+// 250 steps 1880 and 1838; 400 steps 2839 and 2868; 1500 steps 10069 and 10497).
+// Multi-step passes of grids from GRAPH_NODES_MOST nodes on keep ahead of the
+// GPU when launched one by one (one takes 40 us and more, its launches 12-15 us
+// of the host's time): such a call builds no graph for them; a longer one
+// replays the long form (first call of 1500 steps, 1448 x 724: 15.3 against 17.8
+// ms; 4096 x 2048: 55.9 against 56.4).
 constexpr double GRAPH_NODES_MOST = 9e5;
 constexpr int GRAPH_LONG_STEPS = 384;
 // Share of the grid that the kept intermediate states may cover: with more of
@@ -65,7 +66,11 @@ constexpr double MARCH_KEEP_SHARE = 0.25;
 // own, on grids whose single steps are shorter than a link kernel (17 us of
 // latency): one of those a step bounded them (512 x 256 FP32: 10.5 us a step
 // with two link kernels in flight).  The second kind holds nine more states,
-// so it is for states of at most PASS_STATE_BYTES.
+// so it is for states of at most PASS_STATE_BYTES, beyond which they no longer
+// stay in L2 and gain nothing: periodic FP32 1600 x 1100 (63 MB) 84.0 us a step
+// without passes, 86.8 with them, 3000 x 1500 199 and 210, a channel 1500 x 900 with
+// bodies everywhere 57.8 and 63.6, 2200 x 1200 104 and 123; periodic FP16 2048 x 1400
+// 126 and 151; FP64 even (1600 x 900 190.7 and 190.1).
 enum PassKind { PASS_NONE = 0, PASS_MARCH, PASS_STEPS };
 constexpr double PASS_STATE_BYTES = 40e6;
 // Steps of a pass follow one another early (StepArgs::early) up to this many
@@ -513,7 +518,7 @@ cudaError_t launch_one_pass(lbm_ctx *h, int src)
             no_box_sums(a);
             a.step_ctr = h->front + src;
             a.step_off = j;
-        a.pass = 1;
+            a.pass = 1;
             a.next_ctr = j == 0 ? h->front + dst : nullptr;
             a.early = j > 0 && h->tiles_x * h->tiles_y <= EARLY_CTAS * h->sm_count;
             e = launch_collide_stream(h->storage, a, h->tiles_x, h->tiles_y, false, nullptr, h->stream);
