@@ -27,7 +27,7 @@ def work(k):
     lat = binding.Lattice(m, 0.6, 0.05, storage="f16dev", stream=torch.cuda.Stream(), torch_alloc=False)
     start.wait()
     lat.step(1)
-    lat.step(44)
+    lat.step(80)
     launches[k] = lat.launch_count
     out[k] = (lat.populations(), np.stack(lat.force_series("B")))
     lat.close()
@@ -39,7 +39,7 @@ for t in threads:
     t.join()
 for o in out[1:]:
     assert np.array_equal(o[0], out[0][0]) and np.array_equal(o[1], out[0][1])
-assert len(set(launches)) == 1, launches
+assert len(set(launches)) == 1 and launches[0] < 81, launches  # three launches a pass
 print("ok")
 """
 
