@@ -1434,8 +1434,7 @@ lbm_status lbm_prepare(lbm_ctx *h, long n)
             st = build(true, FORM_SHORT, 1);
         if (st == LBM_OK && n > GRAPH_LONG_STEPS) st = build(true, FORM_LONG, 1);
     }
-    if (st != LBM_OK) return st;
-    return LBM_OK;
+    return st;
 }
 
 lbm_status lbm_coefficients(lbm_ctx *h, int scheme, long first, long count, double length, double u_ref,

@@ -1098,8 +1098,7 @@ lbm_status lbm_batch_prepare(lbm_batch *b, long n)
     if (st == LBM_OK && b->pass_ok && n >= first) st = build(true, FORM_FIRST);
     for (int k : {FORM_SHORT, FORM_LONG})
         if (st == LBM_OK && b->pass_ok && n - first >= BATCH_GRAPH_PASSES[k] * GROUP_STEPS) st = build(true, k);
-    if (st != LBM_OK) return st;
-    return LBM_OK;
+    return st;
 }
 
 lbm_status lbm_batch_coefficients(lbm_batch *b, int domain, int scheme, long first, long count, double length,
